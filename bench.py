@@ -97,9 +97,9 @@ KERNELS = {
     "spmv_fp64": ("FS_KERNEL_SPMV_FP64", "k_spmv_full (FP64, refinement residual)"),
     "cheb": ("FS_KERNEL_CHEB", "k_mg (Chebyshev step, finest P2 level, SELL-32)"),
     "assemble": ("FS_KERNEL_ASSEMBLE_CONV", "k_assemble_conv (per-step convection, FP64)"),
-    "cgs_dot": ("FS_KERNEL_CGS_DOT", "k_seg_dot (CGS2 dots h = V^T w, j = 15)"),
-    "cgs_upd": ("FS_KERNEL_CGS_UPD", "k_seg_upd (CGS2 update w -= V h, re-dot, norm; j = 15)"),
-    "cgs_fin": ("FS_KERNEL_CGS_FIN", "k_seg_fin (CGS2 final update and normalisation; j = 15)"),
+    "cgs_dot": ("FS_KERNEL_CGS_DOT", "k_orth_one/k_orth_many, dot pass alone (V^T w and V^T v_j, j = 15)"),
+    "cgs_upd": ("FS_KERNEL_CGS_UPD", "k_orth_one/k_orth_many, update pass with the re-dots alone (j = 15)"),
+    "cgs_fin": ("FS_KERNEL_CGS_FIN", "k_orth_one/k_orth_many, second pass alone (j = 15)"),
 }
 
 

@@ -568,16 +568,18 @@ enum {
                                    the solver arithmetic, timed as a CUDA
                                    graph of `reps` applications; alg_bytes
                                    is 0 (a latency unit of many kernels)   */
-  FS_KERNEL_CGS = 5,            /* one CGS2 orthogonalisation (its three
-                                   passes) at Arnoldi step j = m/2 on the
-                                   Krylov scratch; alg_bytes counts the
-                                   3j + 8 vector sweeps the passes must make
-                                   (each vector once per pass)            */
-  FS_KERNEL_CGS_DOT = 6,        /* its first pass alone (h = V^T w):
+  FS_KERNEL_CGS = 5,            /* one orthogonalisation with both passes taken
+                                   (a step takes the second only when the
+                                   first cancels most of the vector), at
+                                   Arnoldi step j = m/2 on the Krylov
+                                   scratch; alg_bytes counts the 3j + 8
+                                   vector sweeps of dot, update and second
+                                   pass (each vector once per pass)       */
+  FS_KERNEL_CGS_DOT = 6,        /* its dot pass alone (V^T w and V^T v_j):
                                    j + 2 sweeps                           */
-  FS_KERNEL_CGS_UPD = 7,        /* its second pass alone (w -= V h, re-dot,
+  FS_KERNEL_CGS_UPD = 7,        /* its update pass alone (w -= V h, re-dot,
                                    norm): j + 3 sweeps                    */
-  FS_KERNEL_CGS_FIN = 8,        /* its third pass alone (w -= V h2,
+  FS_KERNEL_CGS_FIN = 8,        /* its second pass alone (w -= V h2,
                                    normalise): j + 3 sweeps               */
   FS_PROFILE_COLD_L2 = 0x100    /* flag: L2-cold timing, see above        */
 };

@@ -86,13 +86,15 @@ template <typename V>
 struct Krylov {
   int m = 0;
   int64_t n = 0;
+  int64_t ld = 0;       // distance of the basis vectors: n, padded to 16 bytes
   V* Vb = nullptr;      // (m+1) x n basis
   V* Z = nullptr;       // m x n preconditioned directions
   V* work_p = nullptr;  // nv
   V* work_u = nullptr;  // dim x n2
   V* rhs = nullptr;     // inner right-hand side (precision mode)
   V* sol = nullptr;     // inner solution (precision mode)
-  double* partial = nullptr;  // (m+1) x ntiles
+  double* partial = nullptr;  // one per tile (norms)
+  OrthPlan orth;
   SegState* st = nullptr;
   KCtl* ctl = nullptr;
   cudaGraphExec_t g_check = nullptr, g_iter = nullptr;
@@ -650,17 +652,15 @@ void issue_precond(fs_problem* P, Precision<T>& pr, const DHier<T>& HA, const DH
   }
 }
 
-// Work-list over the n_dof entries: for every instance its vertex and edge
-// ranges in each component block and its pressure range, cut into tiles of
-// at most kTileLen entries; tiles of one instance are consecutive.
-void build_tiles(const fs_problem* P, int sms, std::vector<Tile>& tiles,
-                 std::vector<int>& first, std::vector<int>& count) {
+// The n_dof entries segment by segment: for every instance its vertex and
+// edge ranges in each component block and its pressure range.
+struct Range {
+  int64_t start, len;
+  int seg;
+};
+std::vector<Range> segment_ranges(const fs_problem* P) {
   const Mesh& me = P->mesh->m;
   const int d = P->dim;
-  struct Range {
-    int64_t start, len;
-    int seg;
-  };
   std::vector<Range> ranges;
   for (int s = 0; s < P->nseg; ++s) {
     const Instance& I = me.inst[s];
@@ -670,6 +670,14 @@ void build_tiles(const fs_problem* P, int sms, std::vector<Tile>& tiles,
     }
     ranges.push_back({(int64_t)d * me.n2 + I.voff, I.nv, s});
   }
+  return ranges;
+}
+
+// Work-list over the n_dof entries: the segment ranges cut into tiles of at
+// most kTileLen entries; tiles of one instance are consecutive.
+void build_tiles(const fs_problem* P, int sms, std::vector<Tile>& tiles,
+                 std::vector<int>& first, std::vector<int>& count) {
+  const std::vector<Range> ranges = segment_ranges(P);
   // tile length: one block per tile in the Krylov passes.  With fewer than
   // four tiles of kTileLen per SM the SMs holding one tile more than others
   // set the time, so the count is brought to at most a multiple of the SM
@@ -715,18 +723,106 @@ void build_tiles(const fs_problem* P, int sms, std::vector<Tile>& tiles,
   for (; seg + 1 < P->nseg; ++seg) first[seg + 1] = (int)tiles.size();
 }
 
+// The orthogonalisation kernels' work-lists.  One segment of up to
+// kStreamShare entries per SM: as many blocks as are resident together,
+// unless that leaves a block fewer than kMinShare entries (a barrier over
+// more blocks then costs more than the shorter passes save; FP64 shares go
+// lower, their arithmetic being the longer part).  Else pieces.
+template <typename V>
+int build_orth(fs_problem* P, Krylov<V>& K) {
+  constexpr int64_t kMinShare = sizeof(V) == 4 ? 512 : 128;
+  constexpr int64_t kStreamShare = sizeof(V) == 4 ? 4096 : INT32_MAX / 8;
+  OrthPlan& o = K.orth;
+  const int64_t n = o.n = P->ndof;
+  int64_t cap = orth_blocks<V>(false, &o.smem);
+  const bool many = P->nseg > 1 || n > kStreamShare * cap;
+  if (many) cap = orth_blocks<V>(true, &o.smem);
+  if (cap < 1) {
+    set_error("the orthogonalisation kernel does not fit on this device");
+    return FS_ERR_UNSUPPORTED;
+  }
+  if (!many) {
+    o.blocks = (int)std::max<int64_t>(1, std::min(cap, (n + kMinShare - 1) / kMinShare));
+    o.share = ((n + o.blocks - 1) / o.blocks + 31) / 32 * 32;
+    o.blocks = (int)((n + o.share - 1) / o.share);
+    FS_TRY(P->alloc(&o.partial, (int64_t)128 * o.blocks));
+    o.LU = sizeof(V) == 8 || o.share <= 512 ? 1 : o.share <= 1024 ? 2 : 4;
+  } else {
+    // pieces of one ring chunk; those of a single segment all alike and as
+    // many for every block
+    std::vector<Range> ranges;
+    int64_t piece = kOrthPiece;
+    if (P->nseg == 1) {
+      ranges.push_back({0, n, 0});
+      const int64_t rounds = (n + cap * kOrthPiece - 1) / (cap * kOrthPiece);
+      piece = std::min<int64_t>(kOrthPiece, ((n + cap * rounds - 1) / (cap * rounds) + 31) / 32 * 32);
+    } else {
+      ranges = segment_ranges(P);
+    }
+    std::vector<Tile> pieces;
+    for (const Range& r : ranges)
+      for (int64_t at = 0; at < r.len; at += piece) {
+        Tile t;
+        t.start = r.start + at;
+        t.len = (int32_t)std::min(piece, r.len - at);
+        t.seg = r.seg;
+        pieces.push_back(t);
+      }
+    o.npiece = (int)pieces.size();
+    o.blocks = (int)std::min<int64_t>(cap, o.npiece);
+    // a segment's slots: one per block that holds a piece of it (and per round
+    // of a block's list); its pieces are consecutive and dealt in turn
+    std::vector<int32_t> slot(o.npiece), ss(2 * P->nseg, 0);
+    int32_t next = 0;
+    for (int p = 0; p < o.npiece;) {
+      const int seg = pieces[p].seg, round = p / o.blocks / kOrthList;
+      int e = p;
+      while (e < o.npiece && pieces[e].seg == seg && e / o.blocks / kOrthList == round) {
+        slot[e] = next + (e - p) % o.blocks;
+        ++e;
+      }
+      const int used = std::min(o.blocks, e - p);
+      if (ss[2 * seg + 1] == 0) ss[2 * seg] = next;
+      ss[2 * seg + 1] += used;
+      next += used;
+      p = e;
+    }
+    o.nslot = next;
+    Tile* pc;
+    int32_t *a, *b;
+    FS_TRY(P->upload(&pc, pieces));
+    FS_TRY(P->upload(&a, ss));
+    FS_TRY(P->upload(&b, slot));
+    FS_CUDA(cudaStreamSynchronize(P->stream));  // host sources go out of scope
+    o.pieces = pc;
+    o.seg_slot = a;
+    o.slot = b;
+    FS_TRY(P->alloc(&o.partial, (int64_t)128 * o.nslot));
+  }
+  // threads per group of the dot pass: in FP32 the largest group whose
+  // rounds of 4 entries per thread leave the fewest idle, in FP64 one warp
+  // (its sums over the lanes cost as much as the products they add)
+  const int64_t len = many ? kOrthPiece : o.share;
+  o.T = sizeof(V) == 4 ? 512 : 32;
+  auto slots = [&](int64_t T) { return (len + T * 4 - 1) / (T * 4) * T * 4; };
+  while (o.T > 64 && slots(o.T / 2) < slots(o.T)) o.T /= 2;
+  return FS_OK;
+}
+
 template <typename V>
 int alloc_krylov(fs_problem* P, Krylov<V>& K, int m, const std::vector<int>& first,
                  const std::vector<int>& count) {
   K.m = m;
   K.n = P->ndof;
-  FS_TRY(P->alloc(&K.Vb, (int64_t)(m + 1) * K.n));
+  K.ld = (K.n + 3) / 4 * 4;
+  FS_TRY(P->alloc(&K.Vb, (int64_t)(m + 1) * K.ld));
   FS_TRY(P->alloc(&K.Z, (int64_t)m * K.n));
   FS_TRY(P->alloc(&K.work_p, P->nv));
   FS_TRY(P->alloc(&K.work_u, (int64_t)P->dim * P->n2));
   FS_TRY(P->alloc(&K.rhs, K.n));
   FS_TRY(P->alloc(&K.sol, K.n));
-  FS_TRY(P->alloc(&K.partial, (int64_t)(kMaxRestart + 1) * P->ntiles));
+  FS_TRY(P->alloc(&K.partial, P->ntiles));
+  FS_TRY(build_orth(P, K));
   FS_TRY(P->alloc(&K.st, P->nseg));
   FS_TRY(P->alloc(&K.ctl, 1));
   FS_CUDA(cudaMemsetAsync(K.st, 0, sizeof(SegState) * P->nseg, P->stream));
@@ -738,7 +834,9 @@ int alloc_krylov(fs_problem* P, Krylov<V>& K, int m, const std::vector<int>& fir
   }
   FS_CUDA(cudaMemcpy2DAsync(K.st, sizeof(SegState), init.data(), sizeof(SegHost),
                             sizeof(SegHost), P->nseg, cudaMemcpyHostToDevice, P->stream));
-  KCtl c{m, P->nseg, 0, 0, 0};
+  KCtl c{};
+  c.m = m;
+  c.nseg = P->nseg;
   FS_CUDA(cudaMemcpyAsync(K.ctl, &c, sizeof(KCtl), cudaMemcpyHostToDevice, P->stream));
   FS_CUDA(cudaStreamSynchronize(P->stream));  // host sources go out of scope
   return FS_OK;
@@ -847,19 +945,16 @@ int issue_iter(fs_problem* P, Precision<T>& pr, T* x, int relative_to_beta) {
     FS_CUDA(cudaGraphConditionalHandleCreate(&cond, cg, 0, 0));
   }
   launch_seg_cycle_init(K.st, K.ctl, relative_to_beta, cond, s);
-  launch_seg_scale<T>(K.Vb, tl, K.st, 0, s);
+  launch_seg_scale<T>(K.Vb, tl, K.st, s);
   const int* jp = &K.ctl->j;
   auto step = [&](cudaStream_t q) {
-    const JVec<const T> vj(K.Vb, jp, n);
+    const JVec<const T> vj(K.Vb, jp, K.ld);
     const JVec<T> zj(K.Z, jp, n);
     const JVec<const T> zjc(K.Z, jp, n);
-    const JVec<T> w(K.Vb + n, jp, n);
+    const JVec<T> w(K.Vb + K.ld, jp, K.ld);
     issue_precond<T>(P, pr, pr.HA, pr.HK, vj, zj, P->nseg > 1 ? K.st : nullptr, skip, q);
     launch_spmv_full<T, T>(pr.op, zjc, nullptr, w, 0, skip, q, /*seg=*/true);
-    // one segment: the Givens step rides in the second CGS2 pass
-    const bool fuse = P->nseg == 1;
-    launch_seg_cgs2<T>(K.Vb, n, tl, K.st, K.ctl, K.partial, fuse, cond, q);
-    if (!fuse) launch_seg_givens(K.st, K.ctl, P->nseg, cond, q);
+    launch_seg_orth<T>(K.Vb, K.ld, K.orth, K.st, K.ctl, cond, q);
   };
   if (loop) {
     cudaStreamCaptureStatus cs;
@@ -2584,23 +2679,13 @@ int fs_profile_kernel(fs_problem* P, int kernel, int reps, double* avg_ms, doubl
         auto& K = P->p32.kr;
         FS_TRY(prime(K, &j));
         launch = [P, &K, pass]() {
-          if (pass < 0)
-            launch_seg_cgs2<float>(K.Vb, K.n, P->tl(), K.st, K.ctl, K.partial, false, 0,
-                                   P->stream);
-          else
-            launch_seg_cgs2_pass<float>(K.Vb, K.n, P->tl(), K.st, K.ctl, K.partial, pass,
-                                        P->stream);
+          launch_seg_orth_pass<float>(K.Vb, K.ld, K.orth, K.st, K.ctl, pass, P->stream);
         };
       } else {
         auto& K = P->p64.kr;
         FS_TRY(prime(K, &j));
         launch = [P, &K, pass]() {
-          if (pass < 0)
-            launch_seg_cgs2<double>(K.Vb, K.n, P->tl(), K.st, K.ctl, K.partial, false, 0,
-                                    P->stream);
-          else
-            launch_seg_cgs2_pass<double>(K.Vb, K.n, P->tl(), K.st, K.ctl, K.partial, pass,
-                                         P->stream);
+          launch_seg_orth_pass<double>(K.Vb, K.ld, K.orth, K.st, K.ctl, pass, P->stream);
         };
       }
       // basis vectors each pass must touch, each counted once: dot reads

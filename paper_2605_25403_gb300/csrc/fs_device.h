@@ -492,11 +492,13 @@ struct SegState {
   double rtol;      // set by the host: target of the next cycle, relative to
                     // beta or to bnorm (device data, so captured graphs stay
                     // valid when it changes)
-  double hn;        // ||w|| before normalisation
   unsigned counter[8];
   double H[(kMaxRestart + 1) * kMaxRestart];
   double cs[kMaxRestart], sn[kMaxRestart], g[kMaxRestart + 1];
-  double h2[kMaxRestart + 1];
+  double h2[kMaxRestart + 1];  // coefficients of the running update
+  double f;                    // and 1 / ||w|| (orthogonalisation by pieces),
+  int act;                     // 0: not active, 1: active, 2: second pass needed
+  float E[32 * 32];  // V^T V - I of the cycle's basis (symmetric)
 };
 #ifdef __CUDACC__
 __device__ __forceinline__ bool seg_skipped(const SegSkip& k, int64_t row) {
@@ -512,8 +514,11 @@ struct KCtl {
   int ndone;     // segments done in this cycle
   int all_done;  // every segment done: the spanning kernels skip
   int j;         // Arnoldi step of the cycle (reset by the cycle init,
-                 // advanced by the Givens step: its own kernel, or the
-                 // second CGS2 pass for problems of one segment)
+                 // advanced by the Givens step)
+  int nfin;      // segments whose Givens step of this column is taken
+  int nredo;     // segments whose orthogonalisation needs a second pass
+  unsigned bar, bar_base;  // grid barrier of the orthogonalisation kernel:
+                           // arrivals, and their count before the launch
 };
 
 template <typename V>
@@ -525,23 +530,42 @@ void launch_seg_norm(const V* x, const TileList& tl, SegState* st, double* parti
 void launch_seg_cycle_init(SegState* st, KCtl* ctl, int relative_to_beta,
                            cudaGraphConditionalHandle cond, cudaStream_t s);
 template <typename V>
-void launch_seg_scale(JVec<V> x, const TileList& tl, const SegState* st, int field,
-                      cudaStream_t s);
-// CGS2 on w = V[j + 1] with j = ctl->j, ending with V[j + 1] normalised.
-// with_givens (problems of one segment): the Givens step of column j and the
-// advance of the step index (setting cond when not 0) are done by the
-// second pass, in place of launch_seg_givens.
+void launch_seg_scale(JVec<V> x, const TileList& tl, const SegState* st, cudaStream_t s);
+// How the entries of the n_dof vectors are dealt to the blocks of the
+// orthogonalisation kernels (fs_orth.cu).  share > 0: one segment, block b
+// holds the entries from b share on.  share = 0: pieces of one segment each,
+// dealt to the blocks in turn, a slot of partial sums per piece.
+struct OrthPlan {
+  int blocks = 0;
+  int64_t n = 0;        // entries of a vector
+  int T = 512, LU = 4;  // dot pass: threads per group; update: entries per thread
+  int64_t share = 0;
+  int64_t smem = 0;     // dynamic shared memory, bytes
+  int npiece = 0, nslot = 0;
+  const Tile* pieces = nullptr;
+  const int32_t* slot = nullptr;      // per piece: the slot of its block and segment
+  const int32_t* seg_slot = nullptr;  // per segment: first slot, count
+  double* partial = nullptr;          // 128 per block (share > 0) or per slot
+};
+constexpr int kOrthPiece = 2048;  // entries of a piece at most
+constexpr int kOrthList = 1024;   // pieces a block lists at a time
+// Blocks of the orthogonalisation kernel (the one for pieces when many) that
+// are resident together, and the dynamic shared memory each may use.
 template <typename V>
-void launch_seg_cgs2(V* Vb, int64_t n, const TileList& tl, SegState* st, KCtl* ctl,
-                     double* partial, bool with_givens, cudaGraphConditionalHandle cond,
-                     cudaStream_t s);
-void launch_seg_givens(SegState* st, KCtl* ctl, int nseg, cudaGraphConditionalHandle cond,
-                       cudaStream_t s);
-// One pass of the CGS2 step alone (0: dot, 1: update + re-dot, 2: final
-// update and normalisation; no Givens step), for kernel timing.
+int orth_blocks(bool many, int64_t* smem);
+// Orthogonalises w = V[j + 1] (j = ctl->j; vectors ld apart, a multiple of
+// 4) against V[0..j] and normalises it, takes the Givens step of column j of
+// every active segment and advances the step index (setting cond when not
+// 0).  One cooperative launch.
 template <typename V>
-void launch_seg_cgs2_pass(V* Vb, int64_t n, const TileList& tl, SegState* st, KCtl* ctl,
-                          double* partial, int pass, cudaStream_t s);
+void launch_seg_orth(V* Vb, int64_t ld, const OrthPlan& P, SegState* st, KCtl* ctl,
+                     cudaGraphConditionalHandle cond, cudaStream_t s);
+// For kernel timing, without the Givens step: the orthogonalisation with its
+// second pass always taken (pass < 0), or its dot pass (0), its update pass
+// with the re-dots (1) or its second pass (2) alone.
+template <typename V>
+void launch_seg_orth_pass(V* Vb, int64_t ld, const OrthPlan& P, SegState* st, KCtl* ctl, int pass,
+                          cudaStream_t s);
 template <typename V, typename X>
 void launch_seg_update_x(const SegState* st, const KCtl* ctl, const V* Z, int64_t n,
                          const TileList& tl, X* x, cudaStream_t s);
