@@ -446,8 +446,8 @@ int fs_csr_residual_norm_noalloc(int64_t n, const int64_t* rowptr,
  * re-captured by the next solve); FS_ERR_BUSY while a step is in progress.
  * fs_autotune times one application of the preconditioner (a CUDA graph of
  * `reps` applications, CUDA events) for every pair of candidate thresholds
- * {0, 4096, 16384, 65536} of the velocity and pressure hierarchies and both
- * smoothing group depths, and the saddle-point SpMV (`reps` launches) for
+ * {0, 4096, 16384, 65536} of the velocity and pressure hierarchies and every
+ * smoothing group depth, and the saddle-point SpMV (`reps` launches) for
  * every SpMV group depth, then the persistent form of the preconditioner
  * (persistent_precond = 1) against the best of those; it installs the
  * fastest of each and reports them.  Leaves the state and assembled system
@@ -457,7 +457,9 @@ typedef struct {
   int64_t tail_rows_pressure;
   int32_t spmv_group;    /* SELL slots a thread issues together in the SpMV:
                             4, 6 or 8; 0 = 6 in FP32, 4 in FP64 */
-  int32_t smooth_group;  /* ... in the smoothing passes: 4 or 6; 0 = 4    */
+  int32_t smooth_group;  /* ... in the smoothing passes: 4 or 6; 0 = 8 in
+                            FP32, 4 in FP64 (8 on levels of at most 8
+                            entries a row)                              */
   int32_t coarse_degree; /* degree of the Chebyshev smoother on the levels
                             below the finest (pre and post): 3, 2 or 1;
                             0 = 2 (1: the first step of the restriction is

@@ -210,10 +210,9 @@ struct fs_problem {
   const int32_t* slice_seg_u = nullptr;
   const int32_t* slice_seg_p = nullptr;
   double *natbuf = nullptr, *natbuf2 = nullptr;  // boundary conversions (lazy)
-  // SELL-32 copies of the blocks for the iteration path (slice offsets and
-  // columns shared by both precisions)
-  const int64_t *offA = nullptr, *offB = nullptr, *offBT = nullptr;
-  const int32_t *sciA = nullptr, *sciB = nullptr, *sciBT = nullptr;
+  // SELL-32 copies of the blocks for the iteration path (layouts shared by
+  // both precisions)
+  DSell<double> lA, lB, lBT;  // their layouts (no values)
   double *sA64 = nullptr, *sB64 = nullptr, *sBT64 = nullptr;
   // FP32 data (precision mode)
   float *sA32 = nullptr, *sB32 = nullptr, *sBT32 = nullptr, *diagp32 = nullptr;
@@ -311,14 +310,104 @@ int upload_csr(fs_problem* P, const HostCsr& H, DCsr<T>& d) {
 }
 
 // SELL-32 layout of a CSR pattern: slice offsets (slices of 32 rows, width
-// = the longest row of the slice) and slot-major columns.  Padding slots
-// point at the row itself in a square matrix (a read the row makes anyway)
-// and at column 0 in a rectangular one, so that every column is in range.
+// = the longest row of the slice) and slot-major columns; see DSell for the
+// slices whose columns are runs.  Padding slots of the others point at the
+// row itself in a square matrix and at the row's first column in a
+// rectangular one: reads the row makes anyway.  (In a batch a padding column
+// of another instance would bring in, as 0 x NaN, what that instance's
+// vectors hold once it has converged and is skipped.)
+struct SellLayout {
+  std::vector<int64_t> off;
+  std::vector<int32_t> ci;
+  std::vector<int2> runs;      // per slot (layouts of several widths)
+  std::vector<int32_t> split;  // per slice
+  int64_t width = 0;           // > 0: the width of every slice
+};
+
+// The instance of each row or column of a batch, and where the run of equal
+// instances that holds it ends.
+struct Owners {
+  std::vector<int32_t> own, end;
+  void finish() {
+    end.resize(own.size());
+    for (int64_t i = (int64_t)own.size() - 1; i >= 0; --i)
+      end[i] = i + 1 < (int64_t)own.size() && own[i + 1] == own[i] ? end[i + 1] : (int32_t)i + 1;
+  }
+};
+
+// The column runs of slice rows [r0, r1), width slots, into runs and the
+// columns ci (the slice's first slot); the return value is the slice's split
+// (0: they are no runs).  The rows before the split share at most `width`
+// column offsets between them, and so do the rows after it.  Every column a
+// run implies, also for the padding (coefficient 0), has to lie in the matrix
+// and, with owners (the instance of each row and column of a batch), in the
+// row's own instance.
+int sell_runs(const HostCsr& H, int64_t r0, int64_t r1, int64_t width, const Owners* row_owner,
+              const Owners* col_owner, int2* runs, int32_t* ci) {
+  static thread_local std::vector<int64_t> part[2], merged;
+  part[0].clear();
+  part[1].clear();
+  if (row_owner && row_owner->end[r0] < r1) return 0;
+  int64_t split = 32;
+  int k = 0;
+  for (int64_t r = r0; r < r1; ++r) {
+    merged.clear();
+    const int32_t* c = H.col.data() + H.rowptr[r];
+    const int64_t len = H.rowptr[r + 1] - H.rowptr[r];
+    int64_t b = 0;
+    if (len == (int64_t)part[k].size()) {  // most rows: the offsets of the row before
+      while (b < len && (int64_t)c[b] - (r - r0) == part[k][b]) ++b;
+      if (b == len) continue;
+      b = 0;
+    }
+    size_t a = 0;
+    while (a < part[k].size() || b < len) {  // union of two ascending lists
+      const int64_t x = a < part[k].size() ? part[k][a] : INT64_MAX;
+      const int64_t y = b < len ? (int64_t)c[b] - (r - r0) : INT64_MAX;
+      merged.push_back(std::min(x, y));
+      a += x <= y;
+      b += y <= x;
+    }
+    if ((int64_t)merged.size() <= width) {
+      part[k].swap(merged);
+    } else if (k == 0) {
+      k = 1;
+      split = r - r0;
+      --r;  // the next line starts with this row
+    } else {
+      return 0;
+    }
+  }
+  if (split < 1) return 0;
+  for (int q = 0; q < 2; ++q) {
+    const int64_t t0 = q == 0 ? 0 : split, t1 = q == 0 ? std::min(split, r1 - r0) : r1 - r0;
+    if (t0 >= t1) part[q] = part[0];
+    if (part[q].empty()) part[q].push_back(q == 0 ? 0 : part[0][0]);
+    while ((int64_t)part[q].size() < width) part[q].push_back(part[q].back());
+    for (int64_t t = t0; t < t1; ++t)
+      for (int64_t base : {part[q].front(), part[q].back()}) {
+        const int64_t c = base + t;
+        if (c < 0 || c >= H.ncol) return 0;
+      }
+    if (row_owner)
+      for (int64_t u = 0; u < width && t0 < t1; ++u) {
+        const int64_t c = part[q][u] + t0;
+        if (col_owner->own[c] != row_owner->own[r0] || part[q][u] + t1 > col_owner->end[c]) return 0;
+      }
+  }
+  for (int64_t u = 0; u < width; ++u) {
+    runs[u] = make_int2((int)part[0][u], (int)part[1][u]);
+    for (int64_t t = 0; t < r1 - r0; ++t)
+      ci[32 * u + t] = (int32_t)((t < split ? part[0][u] : part[1][u]) + t);
+  }
+  return (int)split;
+}
+
 // uniform_slack > 0: when padding every slice to the widest costs at most
-// that fraction more slots, all slices get that width; *width receives it
-// (0 when the slices keep their own widths).
-void sell_layout(const HostCsr& H, std::vector<int64_t>& off, std::vector<int32_t>& ci,
-                 double uniform_slack = 0.0, int64_t* width = nullptr) {
+// that fraction more slots, all slices get that width.
+SellLayout sell_layout(const HostCsr& H, double uniform_slack = 0.0,
+                       const Owners* row_owner = nullptr, const Owners* col_owner = nullptr) {
+  SellLayout L;
   const bool square = H.nrow == H.ncol;
   const int64_t n = H.nrow, ns = (n + 31) / 32;
   std::vector<int64_t> ws(ns, 0);
@@ -332,52 +421,79 @@ void sell_layout(const HostCsr& H, std::vector<int64_t>& off, std::vector<int32_
     sum += w;
   }
   const bool uniform = uniform_slack > 0 && ns > 0 && wmax * ns <= (1.0 + uniform_slack) * sum;
-  if (width) *width = uniform ? wmax : 0;
-  off.assign(ns + 1, 0);
-  for (int64_t sl = 0; sl < ns; ++sl) off[sl + 1] = off[sl] + 32 * (uniform ? wmax : ws[sl]);
-  ci.assign(off[ns], 0);
-  for (int64_t r = 0; r < n; ++r) {
-    const int64_t sl = r >> 5, t = r & 31, w = (off[sl + 1] - off[sl]) / 32;
-    const int64_t len = H.rowptr[r + 1] - H.rowptr[r];
-    for (int64_t u = 0; u < w; ++u)
-      ci[off[sl] + 32 * u + t] = u < len ? H.col[H.rowptr[r] + u] : (square ? (int32_t)r : 0);
+  L.width = uniform ? wmax : 0;
+  L.off.assign(ns + 1, 0);
+  for (int64_t sl = 0; sl < ns; ++sl) L.off[sl + 1] = L.off[sl] + 32 * (uniform ? wmax : ws[sl]);
+  L.ci.assign(L.off[ns], 0);
+  if (!uniform) L.runs.assign(L.off[ns] / 32, make_int2(0, 0));
+  L.split.assign(ns, 0);
+  for (int64_t sl = 0; sl < ns; ++sl) {
+    const int64_t r0 = 32 * sl, r1 = std::min(n, r0 + 32), o = L.off[sl], w = (L.off[sl + 1] - o) / 32;
+    if (w == 0) continue;
+    if (!uniform)
+      L.split[sl] = sell_runs(H, r0, r1, w, row_owner, col_owner, &L.runs[o / 32], &L.ci[o]);
+    if (L.split[sl] > 0) continue;
+    for (int64_t r = r0; r < r1; ++r) {
+      const int64_t len = H.rowptr[r + 1] - H.rowptr[r];
+      const int32_t pad = square || len == 0 ? (int32_t)(square ? r : 0) : H.col[H.rowptr[r]];
+      for (int64_t u = 0; u < w; ++u)
+        L.ci[o + 32 * u + (r - r0)] = u < len ? H.col[H.rowptr[r] + u] : pad;
+    }
   }
+  return L;
 }
 
 // Values of a CSR matrix with dimv values per entry (vals, entry-major) in
-// the SELL-32 layout off: component c of slot u of row 32 s + t at
-// (off[s] + 32 u) dimv + 32 c + t; padding slots hold 0.
+// the SELL-32 layout L: component c of slot u of row 32 s + t at
+// (off[s] + 32 u) dimv + 32 c + t; padding slots hold 0.  A row's entries and
+// its slots are both in column order.
 template <typename T>
-std::vector<T> sell_values(const HostCsr& H, const std::vector<int64_t>& off, const double* vals,
-                           int dimv) {
-  std::vector<T> v(off.back() * dimv, T(0));
+std::vector<T> sell_values(const HostCsr& H, const SellLayout& L, const double* vals, int dimv) {
+  std::vector<T> v(L.off.back() * dimv, T(0));
   for (int64_t r = 0; r < H.nrow; ++r) {
-    const int64_t sl = r >> 5, t = r & 31;
-    for (int64_t u = 0; u < H.rowptr[r + 1] - H.rowptr[r]; ++u)
+    const int64_t sl = r >> 5, t = r & 31, w = (L.off[sl + 1] - L.off[sl]) / 32;
+    int64_t k = H.rowptr[r];
+    for (int64_t u = 0; u < w && k < H.rowptr[r + 1]; ++u) {
+      if (L.ci[L.off[sl] + 32 * u + t] != H.col[k]) continue;
       for (int c = 0; c < dimv; ++c)
-        v[(off[sl] + 32 * u) * dimv + 32 * c + t] = (T)vals[(H.rowptr[r] + u) * dimv + c];
+        v[(L.off[sl] + 32 * u) * dimv + 32 * c + t] = (T)vals[k * dimv + c];
+      ++k;
+    }
   }
   return v;
 }
 
+// The layout's arrays on the device (values set by the caller).
 template <typename T>
-int upload_sell(fs_problem* P, const HostCsr& H, DSell<T>& d, double uniform_slack = 0.0) {
-  std::vector<int64_t> off;
-  std::vector<int32_t> ci;
-  int64_t width = 0;
-  sell_layout(H, off, ci, uniform_slack, &width);
-  std::vector<T> v = sell_values<T>(H, off, H.val.data(), 1);
+int upload_layout(fs_problem* P, const HostCsr& H, const SellLayout& L, DSell<T>& d) {
   int64_t* doff;
   int32_t* dci;
-  T* dv;
+  std::vector<int64_t> off = L.off;
+  if (L.width == 0)
+    for (size_t s = 0; s < L.split.size(); ++s) off[s] |= (int64_t)L.split[s] << kSellSplit;
   FS_TRY(P->upload(&doff, off));
-  FS_TRY(P->upload(&dci, ci));
-  FS_TRY(P->upload(&dv, v));
+  FS_TRY(P->upload(&dci, L.ci));
+  if (L.width == 0) {
+    int2* drn;
+    FS_TRY(P->upload(&drn, L.runs));
+    d.runs = drn;
+  }
   d.nrow = H.nrow;
   d.off = doff;
   d.ci = dci;
+  d.width = L.width;
+  return FS_OK;
+}
+
+template <typename T>
+int upload_sell(fs_problem* P, const HostCsr& H, DSell<T>& d, double uniform_slack,
+                const Owners* owner) {
+  const SellLayout L = sell_layout(H, uniform_slack, owner, owner);
+  FS_TRY(upload_layout(P, H, L, d));
+  std::vector<T> v = sell_values<T>(H, L, H.val.data(), 1);
+  T* dv;
+  FS_TRY(P->upload(&dv, v));
   d.v = dv;
-  d.width = width;
   return FS_OK;
 }
 
@@ -482,7 +598,16 @@ int upload_hierarchy(fs_problem* P, const UnionHierarchy& U, int nc, DHier<T>& D
     // level operators: one slice width where padding costs at most 15%
     // more slots (the structured P1 levels); the class-ordered P2 level
     // keeps its per-slice widths
-    FS_TRY(upload_sell<T>(P, hl.A, dl.A, 0.15));
+    const bool batch = l < (int)U.inst_off.size() && U.inst_off[l].size() > 2;
+    Owners owner;  // batches
+    if (batch) {
+      owner.own.resize(hl.A.nrow);
+      for (size_t i = 0; i + 1 < U.inst_off[l].size(); ++i)
+        std::fill(owner.own.begin() + U.inst_off[l][i], owner.own.begin() + U.inst_off[l][i + 1],
+                  (int32_t)i);
+      owner.finish();
+    }
+    FS_TRY(upload_sell<T>(P, hl.A, dl.A, 0.15, batch ? &owner : nullptr));
     if (l + 1 < D.nlev) {
       FS_TRY(upload_csr<T>(P, hl.P, dl.P));
       FS_TRY(upload_csr<T>(P, hl.R, dl.R));
@@ -560,7 +685,7 @@ template <typename T>
 void apply_groups(fs_problem* P, Precision<T>& pr, const fs_schedule& sc) {
   (void)P;
   pr.op.group = sc.spmv_group;
-  pr.HA.group = pr.HK.group = sc.smooth_group ? sc.smooth_group : 4;
+  pr.HA.group = pr.HK.group = sc.smooth_group;
   pr.HA.coarse_deg = pr.HK.coarse_deg = sc.coarse_degree ? sc.coarse_degree : 2;
   pr.HA.fine_deg = pr.HK.fine_deg = sc.fine_degree ? sc.fine_degree : 2;
   const int ratio = sc.cheb_ratio ? sc.cheb_ratio : 8;
@@ -875,9 +1000,12 @@ void set_op(fs_problem* P, DOp<T>& op, const T* A, const T* B, const T* BT, cons
   op.dim = P->dim;
   op.n2 = P->n2;
   op.nv = P->nv;
-  op.A = {P->n2, P->offA, P->sciA, A};
-  op.B = {P->nv, P->offB, P->sciB, B};
-  op.BT = {P->n2, P->offBT, P->sciBT, BT};
+  const auto with = [](const DSell<double>& L, const T* v) {
+    return DSell<T>{L.nrow, L.off, L.ci, v, L.width, L.runs};
+  };
+  op.A = with(P->lA, A);
+  op.B = with(P->lB, B);
+  op.BT = with(P->lBT, BT);
   op.diagp = diagp;
 }
 
@@ -1105,7 +1233,7 @@ int assemble_impl(fs_problem* P, double t_next, const double* w = nullptr,
   launch_bc_rows<double>(P->dm, P->valA, s);
   launch_eval_load(P->dm, P->ph, t_next, 1.0 / P->desc.dt, u_old, P->F, s);
   launch_rhs(P->dm, P->ph, t_next, P->Mv, P->F, P->pinned, P->npinned, P->b, s);
-  launch_csr_to_sell(P->n2, P->dm.rpA, P->valA, P->offA, P->sA64, P->has32 ? P->sA32 : nullptr,
+  launch_csr_to_sell(P->lA, P->dm.rpA, P->dm.ciA, P->valA, P->sA64, P->has32 ? P->sA32 : nullptr,
                      s);
   if (P->sched.schur) assemble_np(P, constw ? nullptr : w, constw ? P->desc.wconst : nullptr);
   FS_TRY(check_launch("assembly"));
@@ -1939,31 +2067,39 @@ int fs_problem_create_batch(fs_mesh* mesh, const fs_problem_desc* descs, int cou
   build_tiles(P.get(), sms, tiles, first, tcount);
   FS_TRY(P->upload(&P->tiles, tiles));
   P->ntiles = (int)tiles.size();
+  Owners oun, opv;  // batches: the instance of each node and vertex
   // SELL-32 blocks of the iteration path: layouts once, B and BT values
   // once (step-invariant), A values scattered after every assembly
   {
-    std::vector<int64_t> oA, oB, oBT;
-    std::vector<int32_t> cA, cB, cBT;
-    sell_layout(me.A, oA, cA);
-    sell_layout(me.B, oB, cB);
-    sell_layout(me.BT, oBT, cBT);
-    int64_t *a, *b, *c;
-    int32_t *ca, *cb, *cc;
-    FS_TRY(P->upload(&a, oA)); FS_TRY(P->upload(&ca, cA));
-    FS_TRY(P->upload(&b, oB)); FS_TRY(P->upload(&cb, cB));
-    FS_TRY(P->upload(&c, oBT)); FS_TRY(P->upload(&cc, cBT));
-    P->offA = a; P->sciA = ca; P->offB = b; P->sciB = cb; P->offBT = c; P->sciBT = cc;
-    FS_TRY(P->alloc(&P->sA64, oA.back()));
-    FS_CUDA(cudaMemsetAsync(P->sA64, 0, sizeof(double) * oA.back(), s));
-    FS_TRY(P->upload(&P->sB64, sell_values<double>(me.B, oB, Bh.data(), dim)));
-    FS_TRY(P->upload(&P->sBT64, sell_values<double>(me.BT, oBT, BTh.data(), dim)));
+    const bool batch = count > 1;
+    if (batch) {
+      oun.own.resize(me.n2);
+      opv.own.resize(me.nv);
+      for (int i = 0; i < count; ++i) {
+        const Instance& I = me.inst[i];
+        for (int64_t q = 0; q < I.nv; ++q) oun.own[I.voff + q] = opv.own[I.voff + q] = i;
+        for (int64_t e = 0; e < I.ne; ++e) oun.own[me.nv + I.eoff + e] = i;
+      }
+      oun.finish();
+      opv.finish();
+    }
+    const Owners *ou = batch ? &oun : nullptr, *op = batch ? &opv : nullptr;
+    const SellLayout LA = sell_layout(me.A, 0.0, ou, ou), LB = sell_layout(me.B, 0.0, op, ou),
+                     LBT = sell_layout(me.BT, 0.0, ou, op);
+    FS_TRY(upload_layout(P.get(), me.A, LA, P->lA));
+    FS_TRY(upload_layout(P.get(), me.B, LB, P->lB));
+    FS_TRY(upload_layout(P.get(), me.BT, LBT, P->lBT));
+    FS_TRY(P->alloc(&P->sA64, LA.off.back()));
+    FS_CUDA(cudaMemsetAsync(P->sA64, 0, sizeof(double) * LA.off.back(), s));
+    FS_TRY(P->upload(&P->sB64, sell_values<double>(me.B, LB, Bh.data(), dim)));
+    FS_TRY(P->upload(&P->sBT64, sell_values<double>(me.BT, LBT, BTh.data(), dim)));
     set_op<double>(P.get(), P->p64.op, P->sA64, P->sB64, P->sBT64, P->diagp);
     if (d0.precision == FS_PREC_FP32_REFINE) {
       P->has32 = true;
-      FS_TRY(P->alloc(&P->sA32, oA.back()));
-      FS_CUDA(cudaMemsetAsync(P->sA32, 0, sizeof(float) * oA.back(), s));
-      FS_TRY(P->upload(&P->sB32, sell_values<float>(me.B, oB, Bh.data(), dim)));
-      FS_TRY(P->upload(&P->sBT32, sell_values<float>(me.BT, oBT, BTh.data(), dim)));
+      FS_TRY(P->alloc(&P->sA32, LA.off.back()));
+      FS_CUDA(cudaMemsetAsync(P->sA32, 0, sizeof(float) * LA.off.back(), s));
+      FS_TRY(P->upload(&P->sB32, sell_values<float>(me.B, LB, Bh.data(), dim)));
+      FS_TRY(P->upload(&P->sBT32, sell_values<float>(me.BT, LBT, BTh.data(), dim)));
       std::vector<float> d32(dp.begin(), dp.end());
       FS_TRY(P->upload(&P->diagp32, d32));
       set_op<float>(P.get(), P->p32.op, P->sA32, P->sB32, P->sBT32, P->diagp32);
@@ -1973,12 +2109,6 @@ int fs_problem_create_batch(fs_mesh* mesh, const fs_problem_desc* descs, int cou
     P->nat = nat;
   }
   if (count > 1) {
-    std::vector<int32_t> own_u(me.n2), own_p(me.nv);
-    for (int i = 0; i < count; ++i) {
-      const Instance& I = me.inst[i];
-      for (int64_t q = 0; q < I.nv; ++q) own_u[I.voff + q] = own_p[I.voff + q] = i;
-      for (int64_t e = 0; e < I.ne; ++e) own_u[me.nv + I.eoff + e] = i;
-    }
     const auto slices = [](const std::vector<int32_t>& own) {
       const int64_t n = (int64_t)own.size(), ns = (n + 31) / 32;
       std::vector<int32_t> ss(ns);
@@ -1991,8 +2121,8 @@ int fs_problem_create_batch(fs_mesh* mesh, const fs_problem_desc* descs, int cou
       return ss;
     };
     int32_t *su, *sp;
-    FS_TRY(P->upload(&su, slices(own_u)));
-    FS_TRY(P->upload(&sp, slices(own_p)));
+    FS_TRY(P->upload(&su, slices(oun.own)));
+    FS_TRY(P->upload(&sp, slices(opv.own)));
     P->slice_seg_u = su;
     P->slice_seg_p = sp;
   }
@@ -2810,7 +2940,7 @@ int fs_autotune(fs_problem* P, int reps, fs_tune_report* report) {
   }
   if (!P->assembled) FS_TRY(assemble_impl(P, P->t + P->desc.dt));
   const int64_t cand[4] = {0, 4096, 16384, 65536};
-  const int sgroups[2] = {4, 6}, pgroups[3] = {4, 6, 8};
+  const int sgroups[3] = {0, 4, 6}, pgroups[3] = {4, 6, 8};
   fs_tune_report r{};
   r.best = P->sched;
   FS_TRY(time_precond(P, reps, P->sched.persistent_precond, &r.default_ms));

@@ -68,7 +68,21 @@ struct DCsr {
 // Sliced ELLPACK with slices of 32 rows (one thread per row): the entries of
 // row 32 s + t sit at off[s] + 32 u + t for the slot u < (off[s+1] - off[s]) / 32,
 // so a warp's loads of one slot are contiguous.  Slots past a row's length
-// hold coefficient 0 and the row itself as column.
+// hold coefficient 0 and a valid column.
+//
+// Columns.  Consecutive rows of a structured mesh have the same stencil
+// shifted by one, so a slice's slots can be laid out by column offset: in a
+// slice with a split > 0 the column of slot u is runs[off / 32 + u].x + t for
+// t < split (the rows of one grid line) and .y + t from there on (those of the
+// next line), 8 bytes per slot instead of 128 and already in L1 for the next
+// slot.  split = 0 (short grid lines, boundary corners): the columns are read
+// from ci, which always holds them.  Which slices qualify is found from the
+// pattern alone.  The split travels in the top byte of the slice's offset,
+// so that it costs no load of its own (a separate array of splits put one
+// more load before the first gather and made the passes on small levels
+// slower); layouts of one width (width > 0, the P1 levels) read no offsets
+// and keep ci (runs = null).
+constexpr int kSellSplit = 56;  // bit position of the split in an offset
 template <typename T>
 struct DSell {
   int64_t nrow = 0;
@@ -78,7 +92,46 @@ struct DSell {
   // > 0: every slice has this many slots (off[s] = 32 s width), so a
   // thread finds its slice without loading off
   int64_t width = 0;
+  const int2* runs = nullptr;
 };
+
+#ifdef __CUDACC__
+// One thread's view of its row: the slice's first slot and slot count, and
+// where the columns come from.
+template <typename T>
+struct SellRow {
+  int64_t first;
+  int w, t, split;
+  __device__ __forceinline__ SellRow(const DSell<T>& A, int64_t row) {
+    const int64_t sl = row >> 5;
+    t = (int)(row & 31);
+    if (A.width) {
+      split = 0;
+      first = sl * 32 * A.width;
+      w = (int)A.width;
+    } else {
+      constexpr int64_t kMask = ((int64_t)1 << kSellSplit) - 1;
+      const int64_t a = A.off[sl], b = A.off[sl + 1];
+      split = (int)(a >> kSellSplit);
+      first = a & kMask;
+      w = (int)(((b & kMask) - first) >> 5);
+    }
+  }
+  // body(col, shift): the column of slot u is col(u) + shift, with shift the
+  // same for every slot (a body adds it to its vector's address once).
+  template <typename F>
+  __device__ __forceinline__ void with_columns(const DSell<T>& A, F body) const {
+    if (split > 0) {
+      const int32_t* __restrict__ q =
+          reinterpret_cast<const int32_t*>(A.runs + (first >> 5)) + (t < split ? 0 : 1);
+      body([q](int u) { return __ldg(q + 2 * u); }, t);
+    } else {
+      const int32_t* __restrict__ q = A.ci + first + t;
+      body([q](int u) { return __ldg(q + 32 * u); }, 0);
+    }
+  }
+};
+#endif
 
 // A vector addressed through the device-side Arnoldi step index: base +
 // (*j) stride (base itself when j is null).  The kernels of one Arnoldi step
@@ -227,10 +280,11 @@ template <typename T, typename V>
 void launch_spmv_full(const DOp<T>& op, JVec<const V> x, const V* b, JVec<V> y,
                       int resid, const int* skip, cudaStream_t s, bool seg = false);
 
-// Scalar CSR values (row pointers rp) into a SELL-32 layout with slice
-// offsets off: out64 (and out32 when not null) receive the n-row matrix.
-void launch_csr_to_sell(int64_t n, const int32_t* rp, const double* in, const int64_t* off,
-                        double* out64, float* out32, cudaStream_t s);
+// Scalar CSR values (row pointers rp, columns ci) into the SELL-32 layout L
+// (its offsets and columns): out64 (and out32 when not null) receive the
+// matrix, zeros in the slots a row does not use.
+void launch_csr_to_sell(const DSell<double>& L, const int32_t* rp, const int32_t* ci,
+                        const double* in, double* out64, float* out32, cudaStream_t s);
 
 // Multigrid level on the device.
 template <typename T>
@@ -267,8 +321,9 @@ struct DHier {
   // the caller's row of block row r, iperm its inverse; null when equal
   const int32_t* perm = nullptr;
   const int32_t* iperm = nullptr;
-  // slots issued together per thread in the smoothing passes (4 or 6)
-  int group = 4;
+  // slots issued together per thread in the smoothing passes (4 or 6; 0: by
+  // precision and level)
+  int group = 0;
   // Chebyshev degree of the pre- and post-smoothing below the finest level
   // and on the finest level (3 or 2 each)
   int coarse_deg = 2;

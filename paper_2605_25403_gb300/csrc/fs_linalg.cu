@@ -43,11 +43,20 @@ __device__ __forceinline__ V group_sum(V v) {
 
 // Row loops take kU slots at a time (loads issued before the FMAs); padding
 // slots have coefficient 0 and a valid column.  The FP32 saddle-point SpMV
-// takes kUSpmv: its rows read more per slot (d gathers, or d values), and
-// deeper groups measured faster there (cube 48^3: 0.115 -> 0.090 ms), while
-// the smoothing pass and the FP64 SpMV are fastest at 4.
+// takes kUSpmv (deeper groups measured faster there, cube 48^3: 0.115 ->
+// 0.090 ms), the FP64 SpMV is fastest at 4; launch_mg has the smoothing
+// passes' rule.
 constexpr int kU = 4;
 constexpr int kUSpmv = 6;
+
+// FP64 FMAs of a partial group's padding are worth a (uniform) branch: at
+// 1/58 of the FP32 rate they are a quarter of a 9-entry row's arithmetic
+// (the saddle-point product of the 33^3 cube 75.0 -> 71.3 us a call).  Not
+// on the P1 levels that take one group of 8: there the branch costs more.
+template <typename V>
+__device__ __forceinline__ constexpr bool skip_padding() {
+  return sizeof(V) == 8;
+}
 
 // ---------------------------------------------------------------------------
 // y = K x  or  y = b - K x with K = [A (per component), -BT; B, diag(D)]
@@ -76,48 +85,53 @@ __global__ void __launch_bounds__(256) k_spmv_full(DOp<T> op, JVec<const V> xv,
 #pragma unroll
     for (int c = 0; c < DIM; ++c) acc[c] = V(0);
     {
-      const int64_t o1 = op.A.off[(row >> 5) + 1];
-      for (int64_t o = op.A.off[row >> 5] + (row & 31); o < o1; o += kUS * 32) {
-        V a[kUS];
-        int32_t j[kUS];
+      const SellRow<T> R(op.A, row);
+      R.with_columns(op.A, [&](auto col, int shift) {
+        const T* __restrict__ v = op.A.v + R.first + R.t;
+        const V* __restrict__ xs = x + shift;
+        for (int k = 0; k < R.w; k += kUS) {
+          V a[kUS], g[kUS][DIM];
 #pragma unroll
-        for (int u = 0; u < kUS; ++u) {
-          const int64_t oo = o + u * 32;
-          const bool ok = oo < o1;
-          a[u] = ok ? (V)op.A.v[oo] : V(0);
-          j[u] = ok ? op.A.ci[oo] : (int32_t)row;
+          for (int u = 0; u < kUS; ++u) {
+            const bool ok = k + u < R.w;
+            a[u] = ok ? (V)v[32 * (k + u)] : V(0);
+            const int32_t j = ok ? col(k + u) : (int32_t)row - shift;
+#pragma unroll
+            for (int c = 0; c < DIM; ++c) g[u][c] = xs[c * n2 + j];
+          }
+#pragma unroll
+          for (int u = 0; u < kUS; ++u) {
+            if (skip_padding<V>() && k + u >= R.w) break;
+#pragma unroll
+            for (int c = 0; c < DIM; ++c) acc[c] += a[u] * g[u][c];
+          }
         }
-        V xv[kUS][DIM];
-#pragma unroll
-        for (int u = 0; u < kUS; ++u)
-#pragma unroll
-          for (int c = 0; c < DIM; ++c) xv[u][c] = x[c * n2 + j[u]];
-#pragma unroll
-        for (int u = 0; u < kUS; ++u)
-#pragma unroll
-          for (int c = 0; c < DIM; ++c) acc[c] += a[u] * xv[u][c];
-      }
+      });
     }
     {
       // d values per slot, component-major: component c of slot u at
       // (slice offset + 32 u) d + 32 c + t
-      const int64_t t32 = row & 31, o1 = op.BT.off[(row >> 5) + 1];
-      for (int64_t o = op.BT.off[row >> 5] + t32; o < o1; o += kU * 32) {
-        V p[kU], bv[kU][DIM];
+      const SellRow<T> R(op.BT, row);
+      R.with_columns(op.BT, [&](auto col, int shift) {
+        const T* __restrict__ v = op.BT.v + R.first * DIM + R.t;
+        const V* __restrict__ ps = xp + shift;
+        for (int k = 0; k < R.w; k += kU) {
+          V p[kU], bv[kU][DIM];
 #pragma unroll
-        for (int u = 0; u < kU; ++u) {
-          const int64_t oo = o + u * 32;
-          const bool ok = oo < o1;
-          const int64_t base = (oo - t32) * DIM + t32;
-          p[u] = ok ? xp[op.BT.ci[oo]] : V(0);
+          for (int u = 0; u < kU; ++u) {
+            const bool ok = k + u < R.w;
+            p[u] = ok ? ps[col(k + u)] : V(0);
 #pragma unroll
-          for (int c = 0; c < DIM; ++c) bv[u][c] = ok ? (V)op.BT.v[base + 32 * c] : V(0);
+            for (int c = 0; c < DIM; ++c) bv[u][c] = ok ? (V)v[32 * ((k + u) * DIM + c)] : V(0);
+          }
+#pragma unroll
+          for (int u = 0; u < kU; ++u) {
+            if (skip_padding<V>() && k + u >= R.w) break;
+#pragma unroll
+            for (int c = 0; c < DIM; ++c) acc[c] -= bv[u][c] * p[u];
+          }
         }
-#pragma unroll
-        for (int u = 0; u < kU; ++u)
-#pragma unroll
-          for (int c = 0; c < DIM; ++c) acc[c] -= bv[u][c] * p[u];
-      }
+      });
     }
 #pragma unroll
     for (int c = 0; c < DIM; ++c) {
@@ -128,45 +142,56 @@ __global__ void __launch_bounds__(256) k_spmv_full(DOp<T> op, JVec<const V> xv,
     const int64_t q = t;
     if (q >= nv || seg_skipped(skp, q)) return;
     V acc = V(0);
-    const int64_t t32 = q & 31, o1 = op.B.off[(q >> 5) + 1];
-    for (int64_t o = op.B.off[q >> 5] + t32; o < o1; o += kUS * 32) {
-      V bv[kUS][DIM], xv[kUS][DIM];
+    const SellRow<T> R(op.B, q);
+    R.with_columns(op.B, [&](auto col, int shift) {
+      const T* __restrict__ v = op.B.v + R.first * DIM + R.t;
+      const V* __restrict__ xs = x + shift;
+      for (int k = 0; k < R.w; k += kUS) {
+        V bv[kUS][DIM], g[kUS][DIM];
 #pragma unroll
-      for (int u = 0; u < kUS; ++u) {
-        const int64_t oo = o + u * 32;
-        const bool ok = oo < o1;
-        const int64_t base = (oo - t32) * DIM + t32;
-        const int32_t j = ok ? op.B.ci[oo] : 0;
+        for (int u = 0; u < kUS; ++u) {
+          const bool ok = k + u < R.w;
+          const int32_t j = ok ? col(k + u) : -shift;
 #pragma unroll
-        for (int c = 0; c < DIM; ++c) {
-          bv[u][c] = ok ? (V)op.B.v[base + 32 * c] : V(0);
-          xv[u][c] = x[c * n2 + j];
+          for (int c = 0; c < DIM; ++c) {
+            bv[u][c] = ok ? (V)v[32 * ((k + u) * DIM + c)] : V(0);
+            g[u][c] = ok ? xs[c * n2 + j] : V(0);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < kUS; ++u) {
+          if (skip_padding<V>() && k + u >= R.w) break;
+#pragma unroll
+          for (int c = 0; c < DIM; ++c) acc += bv[u][c] * g[u][c];
         }
       }
-#pragma unroll
-      for (int u = 0; u < kUS; ++u)
-#pragma unroll
-        for (int c = 0; c < DIM; ++c) acc += bv[u][c] * xv[u][c];
-    }
+    });
     const V v = acc + (V)op.diagp[q] * xp[q];
     const int64_t r = DIM * n2 + q;
     y[r] = resid ? b[r] - v : v;
   }
 }
 
-// CSR -> SELL-32 value scatter, one thread per row.
-__global__ void k_csr_to_sell(int64_t n, const int32_t* __restrict__ rp,
-                              const double* __restrict__ in, const int64_t* __restrict__ off,
+// CSR -> SELL-32 value scatter, one thread per row: the row's entries and its
+// slots are both in column order, so one walk over the slots places them
+// (padding slots, whose column is not the next entry's, get 0).
+__global__ void k_csr_to_sell(DSell<double> L, const int32_t* __restrict__ rp,
+                              const int32_t* __restrict__ ci, const double* __restrict__ in,
                               double* __restrict__ out64, float* __restrict__ out32) {
   const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (r >= n) return;
-  const int64_t base = off[r >> 5] + (r & 31);
-  const int32_t k0 = rp[r], len = rp[r + 1] - k0;
-  for (int32_t u = 0; u < len; ++u) {
-    const double v = in[k0 + u];
-    out64[base + 32 * u] = v;
-    if (out32) out32[base + 32 * u] = (float)v;
-  }
+  if (r >= L.nrow) return;
+  const SellRow<double> R(L, r);
+  const int32_t e = rp[r + 1];
+  const int64_t base = R.first + R.t;
+  R.with_columns(L, [&](auto col, int shift) {
+    int32_t k = rp[r];
+    for (int u = 0; u < R.w; ++u) {
+      double v = 0.0;
+      if (k < e && ci[k] == col(u) + shift) v = in[k++];
+      out64[base + 32 * u] = v;
+      if (out32) out32[base + 32 * u] = (float)v;
+    }
+  });
 }
 
 // ---------------------------------------------------------------------------
@@ -232,39 +257,52 @@ __device__ __forceinline__ void vstore(T* __restrict__ p, const T (&v)[N]) {
   }
 }
 
-// One row of a Chebyshev pass (thread per row on the SELL-32 operator).
-template <typename T, int NC, int NCP, int MODE, int G = kU>
-__device__ __forceinline__ void mg_row(const DSell<T>& A, const T* __restrict__ dinv,
-                                       const T* __restrict__ b, const T* __restrict__ Gin,
-                                       const T* __restrict__ Din, T* __restrict__ Gout,
-                                       T* __restrict__ Dout, T alpha, T beta, T inv_theta,
-                                       T* __restrict__ out, int64_t out_ld,
-                                       const int32_t* __restrict__ perm, int nc, int64_t row) {
-  const int64_t sl = row >> 5;
-  const int64_t o0 = (A.width ? sl * 32 * A.width : A.off[sl]) + (row & 31);
-  const int64_t o1 = A.width ? (sl + 1) * 32 * A.width : A.off[sl + 1];
-  T acc[NCP];
-#pragma unroll
-  for (int c = 0; c < NCP; ++c) acc[c] = T(0);
-  // the slot count is the same for the whole slice: no divergence
-  for (int64_t o = o0; o < o1; o += G * 32) {
-    T a[G];
+// acc += (A x) of one row, x row-major with NCP components.  G slots at a
+// time, their loads before their FMAs; the slot count is the same for the
+// whole slice.  Slots past the last one repeat it with coefficient 0, so that
+// the loads of a partial group are as independent as those of a full one
+// (a branch per slot there chained each column load to its gather).
+template <typename T, int NC, int NCP, int G, typename Col>
+__device__ __forceinline__ void sell_slots(const T* __restrict__ v, int w, Col col,
+                                           const T* __restrict__ x, T (&acc)[NCP]) {
+  for (int k = 0; k < w; k += G) {
+    T a[G], g[G][NCP];
     int32_t j[G];
 #pragma unroll
+    for (int u = 0; u < G; ++u) a[u] = k + u < w ? v[32 * (k + u)] : T(0);
+#pragma unroll
+    for (int u = 0; u < G; ++u) j[u] = col(k + u < w ? k + u : k);
+#pragma unroll
+    for (int u = 0; u < G; ++u) vload<T, NCP>(x + (int64_t)j[u] * NCP, g[u]);
+#pragma unroll
     for (int u = 0; u < G; ++u) {
-      const int64_t oo = o + u * 32;
-      const bool ok = oo < o1;
-      a[u] = ok ? A.v[oo] : T(0);
-      j[u] = ok ? A.ci[oo] : (int32_t)row;
-    }
-    T g[G][NCP];
-#pragma unroll
-    for (int u = 0; u < G; ++u) vload<T, NCP>(Gin + (int64_t)j[u] * NCP, g[u]);
-#pragma unroll
-    for (int u = 0; u < G; ++u)
+      if (skip_padding<T>() && G < 8 && k + u >= w) break;
 #pragma unroll
       for (int c = 0; c < NC; ++c) acc[c] += a[u] * g[u][c];
+    }
   }
+}
+
+template <typename T, int NC, int NCP, int G>
+__device__ __forceinline__ void sell_row_times(const DSell<T>& A, const T* __restrict__ x,
+                                               int64_t row, T (&acc)[NCP]) {
+  const SellRow<T> R(A, row);
+  const T* __restrict__ v = A.v + R.first + R.t;
+#pragma unroll
+  for (int c = 0; c < NCP; ++c) acc[c] = T(0);
+  R.with_columns(A, [&](auto col, int shift) {
+    sell_slots<T, NC, NCP, G>(v, R.w, col, x + shift * NCP, acc);
+  });
+}
+
+// The row's own part of a Chebyshev pass: acc = (A Gin) of the row.
+template <typename T, int NC, int NCP, int MODE>
+__device__ __forceinline__ void mg_finish(const T (&acc)[NCP], const T* __restrict__ dinv,
+                                          const T* __restrict__ b, const T* __restrict__ Gin,
+                                          const T* __restrict__ Din, T* __restrict__ Gout,
+                                          T* __restrict__ Dout, T alpha, T beta, T inv_theta,
+                                          T* __restrict__ out, int64_t out_ld,
+                                          const int32_t* __restrict__ perm, int nc, int64_t row) {
   T gx[NCP], d[NCP], bb[NCP];
   vload<T, NCP>(Gin + row * NCP, gx);
   if (MODE == MG_STEP || MODE == MG_LAST) vload<T, NCP>(Din + row * NCP, d);
@@ -298,6 +336,20 @@ __device__ __forceinline__ void mg_row(const DSell<T>& A, const T* __restrict__ 
   }
   vstore<T, NCP>(Gout + row * NCP, go);
   if (MODE == MG_STEP || MODE == MG_START) vstore<T, NCP>(Dout + row * NCP, dout);
+}
+
+// One row of a Chebyshev pass (thread per row on the SELL-32 operator).
+template <typename T, int NC, int NCP, int MODE, int G = kU>
+__device__ __forceinline__ void mg_row(const DSell<T>& A, const T* __restrict__ dinv,
+                                       const T* __restrict__ b, const T* __restrict__ Gin,
+                                       const T* __restrict__ Din, T* __restrict__ Gout,
+                                       T* __restrict__ Dout, T alpha, T beta, T inv_theta,
+                                       T* __restrict__ out, int64_t out_ld,
+                                       const int32_t* __restrict__ perm, int nc, int64_t row) {
+  T acc[NCP];
+  sell_row_times<T, NC, NCP, G>(A, Gin, row, acc);
+  mg_finish<T, NC, NCP, MODE>(acc, dinv, b, Gin, Din, Gout, Dout, alpha, beta, inv_theta, out,
+                              out_ld, perm, nc, row);
 }
 
 // Restriction row (L lanes; every lane of the group calls it, `active`
@@ -685,20 +737,31 @@ void launch_mg(int mode, const DLevel<T>& L, const T* b, const T* Gin, const T* 
   const int64_t n = L.A.nrow;
   const T it = (T)L.inv_theta;
   constexpr int NC = NCP == 4 ? 3 : NCP;  // real components (3D pads 3 to 4)
+  // slots per group: the schedule's, else 8 in FP32 and 4 in FP64 (8 on
+  // levels of at most 8 slots a row, one group: the 2D P1 grids).  Inside the
+  // restart loop, with a level's operator coming from L2 or HBM, 8 against 4
+  // in FP32: one application of the preconditioner 52.9 -> 43.4 us on the 7^3
+  // cube, 50.7 -> 44.2 on the 32^2 square, 320 -> 310 on the 48^3 cube, 80.4
+  // -> 75.1 on the channel; FP64 rows are partly bound by their arithmetic
+  // (256x48 channel 112 -> 115 us at 8 everywhere).  Threads per block: 128
+  // in FP64 (112 -> 109 us), no difference in FP32.
+  constexpr bool f32 = std::is_same<T, float>::value;
+  const int g = group ? group : f32 || (L.A.width > 0 && L.A.width <= 8) ? 8 : 4;
+  constexpr int kB = f32 ? 256 : 128;
 #define FS_MG(M, G)                                                                        \
-  launch_k(k_mg<T, NC, NCP, M, G>, blocks_for(n), 256, 0, s, L.A, L.dinv, b, Gin, Din, Gout,    \
+  launch_k(k_mg<T, NC, NCP, M, G>, blocks_for(n, kB), kB, 0, s, L.A, L.dinv, b, Gin, Din, Gout, \
            Dout, alpha, beta, it, out, out_ld, perm, nc, L.skip, skip)
-  if (group == 6) {
-    if (mode == MG_STEP) FS_MG(MG_STEP, 6);
-    else if (mode == MG_RESID) FS_MG(MG_RESID, 6);
-    else if (mode == MG_START) FS_MG(MG_START, 6);
-    else FS_MG(MG_LAST, 6);
-  } else {
-    if (mode == MG_STEP) FS_MG(MG_STEP, 4);
-    else if (mode == MG_RESID) FS_MG(MG_RESID, 4);
-    else if (mode == MG_START) FS_MG(MG_START, 4);
-    else FS_MG(MG_LAST, 4);
-  }
+#define FS_MG_MODES(G)                              \
+  do {                                              \
+    if (mode == MG_STEP) FS_MG(MG_STEP, G);         \
+    else if (mode == MG_RESID) FS_MG(MG_RESID, G);  \
+    else if (mode == MG_START) FS_MG(MG_START, G);  \
+    else FS_MG(MG_LAST, G);                         \
+  } while (0)
+  if (g == 8) FS_MG_MODES(8);
+  else if (g == 6) FS_MG_MODES(6);
+  else FS_MG_MODES(4);
+#undef FS_MG_MODES
 #undef FS_MG
   count_launches(1);
 }
@@ -876,26 +939,24 @@ __global__ void __launch_bounds__(256) k_mg_first1(DSell<T> A, const T* __restri
   const int64_t row = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (row >= A.nrow || seg_skipped(sk, row)) return;
   const T* __restrict__ r = rv.get();
-  const int64_t sl = row >> 5;
-  const int64_t o0 = (A.width ? sl * 32 * A.width : A.off[sl]) + (row & 31);
-  const int64_t o1 = A.width ? (sl + 1) * 32 * A.width : A.off[sl + 1];
+  const SellRow<T> R(A, row);
   T acc = T(0);
-  for (int64_t o = o0; o < o1; o += G * 32) {
-    T a[G];
-    int32_t j[G];
+  R.with_columns(A, [&](auto col, int shift) {
+    const T* __restrict__ v = A.v + R.first + R.t;
+    const T *__restrict__ ds = dinv + shift, *__restrict__ rs = r + shift;
+    for (int k = 0; k < R.w; k += G) {
+      T a[G], g[G];
 #pragma unroll
-    for (int u = 0; u < G; ++u) {
-      const int64_t oo = o + u * 32;
-      const bool ok = oo < o1;
-      a[u] = ok ? A.v[oo] : T(0);
-      j[u] = ok ? A.ci[oo] : (int32_t)row;
+      for (int u = 0; u < G; ++u) {
+        const bool ok = k + u < R.w;
+        a[u] = ok ? v[32 * (k + u)] : T(0);
+        const int32_t j = ok ? col(k + u) : (int32_t)row - shift;
+        g[u] = ds[j] * rs[j] * inv_theta;
+      }
+#pragma unroll
+      for (int u = 0; u < G; ++u) acc += a[u] * g[u];
     }
-    T g[G];
-#pragma unroll
-    for (int u = 0; u < G; ++u) g[u] = dinv[j[u]] * r[j[u]] * inv_theta;
-#pragma unroll
-    for (int u = 0; u < G; ++u) acc += a[u] * g[u];
-  }
+  });
   const T v = r[row], di = dinv[row];
   const T g0 = di * v * inv_theta;
   const T d = alpha * g0 + beta * di * (v - acc);
@@ -973,13 +1034,30 @@ __global__ void __launch_bounds__(256) k_bt_add_mg(DSell<T> BT, int64_t n2, int6
   T acc[DIM];
 #pragma unroll
   for (int c = 0; c < DIM; ++c) acc[c] = T(0);
-  const int64_t o1 = BT.off[(row >> 5) + 1];
-  for (int64_t o = BT.off[row >> 5] + (row & 31); o < o1; o += 32) {
-    const int64_t base = (o - (row & 31)) * DIM + (row & 31);
-    const T p = ZREAD ? zp[BT.ci[o]] : cc_combine(mpl, rp, yk, inv_dt, BT.ci[o]);
+  const SellRow<T> R(BT, row);
+  R.with_columns(BT, [&](auto col, int shift) {
+    const T* __restrict__ v = BT.v + R.first * DIM + R.t;
+    for (int k = 0; k < R.w; k += kU) {
+      T p[kU], bv[kU][DIM];
 #pragma unroll
-    for (int c = 0; c < DIM; ++c) acc[c] += BT.v[base + 32 * c] * p;
-  }
+      for (int u = 0; u < kU; ++u) {
+        p[u] = T(0);
+        if (k + u < R.w) {
+          const int32_t j = col(k + u) + shift;
+          p[u] = ZREAD ? zp[j] : cc_combine(mpl, rp, yk, inv_dt, j);
+#pragma unroll
+          for (int c = 0; c < DIM; ++c) bv[u][c] = v[32 * ((k + u) * DIM + c)];
+        } else {
+#pragma unroll
+          for (int c = 0; c < DIM; ++c) bv[u][c] = T(0);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u)
+#pragma unroll
+        for (int c = 0; c < DIM; ++c) acc[c] += bv[u][c] * p[u];
+    }
+  });
   T tv[NCP], d0[NCP];
   const T sc = dinv0 ? dinv0[dst] * inv_theta0 : T(0);
 #pragma unroll
@@ -1123,9 +1201,9 @@ template void launch_spmv_full<double, double>(const DOp<double>&, JVec<const do
 template void launch_spmv_full<float, float>(const DOp<float>&, JVec<const float>, const float*,
                                              JVec<float>, int, const int*, cudaStream_t, bool);
 
-void launch_csr_to_sell(int64_t n, const int32_t* rp, const double* in, const int64_t* off,
-                        double* out64, float* out32, cudaStream_t s) {
-  k_csr_to_sell<<<blocks_for(n), 256, 0, s>>>(n, rp, in, off, out64, out32);
+void launch_csr_to_sell(const DSell<double>& L, const int32_t* rp, const int32_t* ci,
+                        const double* in, double* out64, float* out32, cudaStream_t s) {
+  k_csr_to_sell<<<blocks_for(L.nrow), 256, 0, s>>>(L, rp, ci, in, out64, out32);
   count_launches(1);
 }
 
@@ -1170,12 +1248,10 @@ void launch_precond(const DOp<T>& op, const DHier<T>& HA, const DHier<T>& HK,
     const bool k1 = HK.nlev > 1;
     const DLevel<T>& L0 = HK.lev[0];
     if (k1 && HK.tail != 0 && !HK.perm && HK.fine_deg != 1) {
-      if (HK.group == 6)
-        launch_k(k_mg_first1<T, 6>, blocks_for(nv), 256, 0, s, L0.A, L0.dinv, rp,
-                 (T)L0.inv_theta, (T)L0.a1, (T)L0.b1, HK.b[0], HK.G1[0], HK.D1[0], L0.skip, skip);
-      else
-        launch_k(k_mg_first1<T, 4>, blocks_for(nv), 256, 0, s, L0.A, L0.dinv, rp,
-                 (T)L0.inv_theta, (T)L0.a1, (T)L0.b1, HK.b[0], HK.G1[0], HK.D1[0], L0.skip, skip);
+      auto k = HK.group == 6 ? k_mg_first1<T, 6> : HK.group == 4 ? k_mg_first1<T, 4>
+                                                                 : k_mg_first1<T, 8>;
+      launch_k(k, blocks_for(nv), 256, 0, s, L0.A, L0.dinv, rp, (T)L0.inv_theta, (T)L0.a1,
+               (T)L0.b1, HK.b[0], HK.G1[0], HK.D1[0], L0.skip, skip);
       count_launches(1);
       vcycle_level<T, 1>(HK, 0, JVec<T>(work_p), nv, 1, skip, s, /*first_done=*/true);
     } else {
@@ -1403,8 +1479,9 @@ __device__ __forceinline__ void flow_item(const FlowArgs<T>& a, const FlowPhase<
         T acc[DIM];
 #pragma unroll
         for (int c = 0; c < DIM; ++c) acc[c] = T(0);
-        const int64_t o1 = a.BT.off[(row >> 5) + 1];
-        for (int64_t o = a.BT.off[row >> 5] + (row & 31); o < o1; o += 32) {
+        const SellRow<T> R(a.BT, row);
+        const int64_t o1 = R.first + 32 * (int64_t)R.w;
+        for (int64_t o = R.first + R.t; o < o1; o += 32) {
           const int64_t base = (o - (row & 31)) * DIM + (row & 31);
           const T p = zp[a.BT.ci[o]];
 #pragma unroll
