@@ -194,9 +194,12 @@ struct fs_problem {
   // increment, right-hand side and CG vectors (velocity-sized), inverse
   // diagonals of the three operators, partials, CG scalars, fixed vertices
   double *ip_us = nullptr, *ip_dp = nullptr, *ip_rhs = nullptr, *ip_r = nullptr;
-  double *ip_z = nullptr, *ip_p = nullptr, *ip_q = nullptr;
+  double *ip_z = nullptr, *ip_p = nullptr, *ip_p2 = nullptr, *ip_q = nullptr;
   double *ip_dA = nullptr, *ip_dM = nullptr, *ip_dK = nullptr, *ip_part = nullptr;
   double *ip_sc = nullptr, *ip_nrm = nullptr;
+  CgCtl* ip_ctl = nullptr;
+  // SELL-32 values of the two velocity operators (P2/P1 problems)
+  double *ip_sA = nullptr, *ip_sM = nullptr;
   uint8_t* ip_fixed = nullptr;
   // pressure stage preconditioned by a V-cycle of the pressure Laplacian
   // hierarchy (P2/P1 problems): old residual, FP32 copies for an FP32 hierarchy
@@ -213,6 +216,7 @@ struct fs_problem {
   // SELL-32 copies of the blocks for the iteration path (layouts shared by
   // both precisions)
   DSell<double> lA, lB, lBT;  // their layouts (no values)
+  int64_t sA_slots = 0;       // value slots of lA
   double *sA64 = nullptr, *sB64 = nullptr, *sBT64 = nullptr;
   // FP32 data (precision mode)
   float *sA32 = nullptr, *sB32 = nullptr, *sBT32 = nullptr, *diagp32 = nullptr;
@@ -2089,6 +2093,7 @@ int fs_problem_create_batch(fs_mesh* mesh, const fs_problem_desc* descs, int cou
     FS_TRY(upload_layout(P.get(), me.A, LA, P->lA));
     FS_TRY(upload_layout(P.get(), me.B, LB, P->lB));
     FS_TRY(upload_layout(P.get(), me.BT, LBT, P->lBT));
+    P->sA_slots = LA.off.back();
     FS_TRY(P->alloc(&P->sA64, LA.off.back()));
     FS_CUDA(cudaMemsetAsync(P->sA64, 0, sizeof(double) * LA.off.back(), s));
     FS_TRY(P->upload(&P->sB64, sell_values<double>(me.B, LB, Bh.data(), dim)));
@@ -2463,14 +2468,15 @@ int fs_solve_steady(fs_problem* P, const fs_solve_opts* opts, double nl_tol, int
 static int ipcs_setup(fs_problem* P) {
   if (P->ip_us) return FS_OK;
   const int64_t nvel = (int64_t)P->dim * P->n2, nv = P->nv;
-  for (double** v : {&P->ip_us, &P->ip_rhs, &P->ip_r, &P->ip_z, &P->ip_p, &P->ip_q, &P->ip_dA,
-                     &P->ip_dM})
+  for (double** v : {&P->ip_us, &P->ip_rhs, &P->ip_r, &P->ip_z, &P->ip_p, &P->ip_p2, &P->ip_q,
+                     &P->ip_dA, &P->ip_dM})
     FS_TRY(P->alloc(v, nvel));
   FS_TRY(P->alloc(&P->ip_dp, nv));
   FS_TRY(P->alloc(&P->ip_dK, nv));
   FS_TRY(P->alloc(&P->ip_part, ipcs_part_size(P->dm)));
   FS_TRY(P->alloc(&P->ip_sc, 4));
   FS_TRY(P->alloc(&P->ip_nrm, diff_norms_scratch()));
+  FS_TRY(P->alloc(&P->ip_ctl, 1));
   std::vector<uint8_t> fixed(nv, 0);
   for (int32_t q : P->pinned_host) fixed[q] = 1;
   FS_TRY(P->upload(&P->ip_fixed, fixed));
@@ -2487,6 +2493,13 @@ static int ipcs_setup(fs_problem* P) {
     }
   }
   cudaStream_t s = P->stream;
+  if (!P->p3) {
+    const int64_t slots = P->sA_slots;
+    FS_TRY(P->alloc(&P->ip_sA, slots));
+    FS_TRY(P->alloc(&P->ip_sM, slots));
+    launch_csr_to_sell(P->lA, P->dm.rpA, P->dm.ciA, P->baseA, P->ip_sA, nullptr, s);
+    launch_csr_to_sell(P->lA, P->dm.rpA, P->dm.ciA, P->Mv, P->ip_sM, nullptr, s);
+  }
   launch_ipcs_dinv(P->dm, 0, P->baseA, nullptr, P->ip_dA, s);
   launch_ipcs_dinv(P->dm, 0, P->Mv, nullptr, P->ip_dM, s);
   launch_ipcs_dinv(P->dm, 1, P->Kp, P->ip_fixed, P->ip_dK, s);
@@ -2514,24 +2527,44 @@ static void ipcs_vcycle(fs_problem* P, const double* r, double* z) {
 // P3/P2 pressure take Jacobi preconditioning; the P2/P1 pressure stage takes
 // one V-cycle per iteration in flexible CG (Polak-Ribiere beta), which keeps
 // the iteration count flat in the mesh size.
-static int ipcs_cg(fs_problem* P, int which, const double* vals, const double* dinv,
-                   const double* rhs, double* x, double rtol, int max_iter, int* iters,
-                   double* relres) {
+static int ipcs_cg(fs_problem* P, int which, const double* vals, const double* sell,
+                   const double* dinv, const double* rhs, double* x, double rtol, int max_iter,
+                   int* iters, double* relres) {
   cudaStream_t s = P->stream;
   const DMesh& m = P->dm;
   const int64_t n = which == 1 ? P->nv : (int64_t)P->dim * P->n2;
   const uint8_t* fixed = which == 1 ? P->ip_fixed : nullptr;
-  const bool mg = which == 1 && P->ip_mg;
   launch_ipcs_fix(m, which, fixed, rhs, x, s);
+  if (which != 1 || !P->ip_mg) {
+    CgOp op;
+    op.n = which == 1 ? P->nv : P->n2;
+    op.fixed = which == 1 ? P->ip_fixed : m.dirichlet;
+    if (sell) {
+      op.sell = P->lA;
+      op.sell.v = sell;
+    }
+    op.rp = which == 1 ? m.rpK : m.rpA;
+    op.ci = which == 1 ? m.ciK : m.ciA;
+    op.v = vals;
+    launch_cg_solve(m, which, op, rhs, x, dinv, P->ip_r, P->ip_z, P->ip_p, P->ip_p2, P->ip_q,
+                    P->ip_part, P->ip_ctl, rtol, max_iter, s);
+    FS_TRY(check_launch("ipcs cg"));
+    CgCtl c;
+    FS_CUDA(cudaMemcpyAsync(&c, P->ip_ctl, sizeof(c), cudaMemcpyDeviceToHost, s));
+    FS_CUDA(cudaStreamSynchronize(s));
+    *iters = c.iters;
+    *relres = c.bb > 0 ? std::sqrt(c.rr / c.bb) : std::sqrt(c.rr);
+    if (c.bad) return FS_ERR_TIMEOUT;
+    if (!std::isfinite(*relres)) return FS_ERR_NUMERIC;
+    return *relres <= 100.0 * rtol ? FS_OK : FS_ERR_NOT_CONVERGED;
+  }
   launch_diff_norms(rhs, rhs, n, P->ip_nrm, s);
   launch_ipcs_apply(m, which, vals, fixed, x, P->ip_q, nullptr, s);
   launch_cg_init(n, rhs, P->ip_q, dinv, P->ip_r, P->ip_z, P->ip_p, P->ip_part, P->ip_sc, s);
-  if (mg) {
-    ipcs_vcycle(P, P->ip_r, P->ip_z);
-    launch_cg_dots_flex(n, fixed, P->ip_r, P->ip_t, P->ip_z, P->ip_p, 1, P->ip_part, P->ip_sc, s);
-  }
+  ipcs_vcycle(P, P->ip_r, P->ip_z);
+  launch_cg_dots_flex(n, fixed, P->ip_r, P->ip_t, P->ip_z, P->ip_p, 1, P->ip_part, P->ip_sc, s);
   FS_TRY(check_launch("ipcs cg init"));
-  double h[4] = {0, 0, 0, 0};
+  double h[6] = {0, 0, 0, 0, 0, 0};
   FS_CUDA(cudaMemcpyAsync(h, P->ip_nrm, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
   FS_CUDA(cudaMemcpyAsync(h + 2, P->ip_sc, 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
   FS_CUDA(cudaStreamSynchronize(s));
@@ -2543,15 +2576,10 @@ static int ipcs_cg(fs_problem* P, int which, const double* vals, const double* d
     for (int c = 0; c < 8 && it < max_iter; ++c, ++it) {
       const int nb = launch_ipcs_apply(m, which, vals, fixed, P->ip_p, P->ip_q, P->ip_part, s);
       launch_cg_alpha(P->ip_part, nb, P->ip_sc, s);
-      if (mg) {
-        launch_cg_update_flex(n, P->ip_sc, P->ip_p, P->ip_q, x, P->ip_r, P->ip_t, P->ip_part, s);
-        ipcs_vcycle(P, P->ip_r, P->ip_z);
-        launch_cg_dots_flex(n, fixed, P->ip_r, P->ip_t, P->ip_z, P->ip_p, 0, P->ip_part,
-                            P->ip_sc, s);
-      } else {
-        launch_cg_update(n, P->ip_sc, P->ip_p, P->ip_q, dinv, x, P->ip_r, P->ip_z, P->ip_part,
-                         s);
-      }
+      launch_cg_update_flex(n, P->ip_sc, P->ip_p, P->ip_q, x, P->ip_r, P->ip_t, P->ip_part, s);
+      ipcs_vcycle(P, P->ip_r, P->ip_z);
+      launch_cg_dots_flex(n, fixed, P->ip_r, P->ip_t, P->ip_z, P->ip_p, 0, P->ip_part, P->ip_sc,
+                          s);
       launch_cg_dir(n, P->ip_sc, P->ip_z, P->ip_p, s);
     }
     FS_TRY(check_launch("ipcs cg"));
@@ -2581,21 +2609,21 @@ static int ipcs_step_impl(fs_problem* P, double rtol, int max_iter, fs_ipcs_stat
   // stage 1: tentative velocity, from u^n
   launch_ipcs_rhs1(P->dm, P->valA, P->baseA, P->BT, P->b, P->x, P->ip_rhs, s);
   FS_CUDA(cudaMemcpyAsync(P->ip_us, P->x, sizeof(double) * nvel, cudaMemcpyDeviceToDevice, s));
-  int rc = ipcs_cg(P, 0, P->baseA, P->ip_dA, P->ip_rhs, P->ip_us, rtol, max_iter, &st->iters[0],
-                   &st->rel_res[0]);
+  int rc = ipcs_cg(P, 0, P->baseA, P->ip_sA, P->ip_dA, P->ip_rhs, P->ip_us, rtol, max_iter,
+                   &st->iters[0], &st->rel_res[0]);
   // stage 2: pressure increment, from 0
   if (rc == FS_OK) {
     launch_ipcs_rhs2(P->dm, P->B, P->ip_us, 1.0 / dt, P->ip_fixed, P->b, P->x, P->ip_rhs, s);
     FS_CUDA(cudaMemsetAsync(P->ip_dp, 0, sizeof(double) * P->nv, s));
-    rc = ipcs_cg(P, 1, P->Kp, P->ip_dK, P->ip_rhs, P->ip_dp, rtol, max_iter, &st->iters[1],
-                 &st->rel_res[1]);
+    rc = ipcs_cg(P, 1, P->Kp, nullptr, P->ip_dK, P->ip_rhs, P->ip_dp, rtol, max_iter,
+                 &st->iters[1], &st->rel_res[1]);
   }
   // stage 3: corrected velocity, from u*; then p^{n+1} = p^n + dp
   if (rc == FS_OK) {
     launch_ipcs_rhs3(P->dm, P->Mv, P->BT, P->b, P->ip_us, P->ip_dp, dt, P->ip_rhs, s);
     FS_CUDA(cudaMemcpyAsync(P->x, P->ip_us, sizeof(double) * nvel, cudaMemcpyDeviceToDevice, s));
-    rc = ipcs_cg(P, 0, P->Mv, P->ip_dM, P->ip_rhs, P->x, rtol, max_iter, &st->iters[2],
-                 &st->rel_res[2]);
+    rc = ipcs_cg(P, 0, P->Mv, P->ip_sM, P->ip_dM, P->ip_rhs, P->x, rtol, max_iter,
+                 &st->iters[2], &st->rel_res[2]);
     launch_ipcs_add(P->nv, P->ip_dp, P->x + nvel, s);
     FS_TRY(check_launch("ipcs pressure update"));
   }

@@ -492,14 +492,33 @@ void launch_ipcs_fix(const DMesh& m, int which, const uint8_t* fixed, const doub
 void launch_ipcs_add(int64_t n, const double* x, double* y, cudaStream_t s);
 // doubles of block-partial scratch the CG kernels need on this mesh
 int ipcs_part_size(const DMesh& m);
-// Jacobi-preconditioned CG steps; sc (4 doubles on the device): rz, alpha,
-// beta, rr.
+// A whole Jacobi-preconditioned CG solve of the stage `which` (0: DIM
+// components, 1: pressure) as one cooperative launch: op the operator, x the
+// guess with its fixed unknowns in place, dinv the inverse diagonal, part
+// ipcs_part_size doubles; ctl receives the iterations, the squared norms of
+// the true residual and of rhs, and bad = 1 when a wait ran out.
+constexpr int kCgMaxBlocks = 256;
+struct CgCtl {
+  unsigned bar;
+  int iters, bad, pad;
+  double rr, bb;
+};
+struct CgOp {
+  int64_t n = 0;                   // rows
+  const uint8_t* fixed = nullptr;  // identity rows
+  DSell<double> sell;              // used when its values are set, else CSR:
+  const int32_t *rp = nullptr, *ci = nullptr;
+  const double* v = nullptr;
+};
+void launch_cg_solve(const DMesh& m, int which, const CgOp& op, const double* rhs, double* x,
+                     const double* dinv, double* r, double* z, double* p, double* p2,
+                     double* q, double* part, CgCtl* ctl, double rtol, int max_iter,
+                     cudaStream_t s);
+// The V-cycle-preconditioned pressure stage, a kernel per step; sc (4 doubles
+// on the device): rz, alpha, beta, rr.
 void launch_cg_init(int64_t n, const double* rhs, const double* y, const double* dinv, double* r,
                     double* z, double* p, double* part, double* sc, cudaStream_t s);
 void launch_cg_alpha(const double* part, int nb, double* sc, cudaStream_t s);
-void launch_cg_update(int64_t n, double* sc, const double* p, const double* q,
-                      const double* dinv, double* x, double* r, double* z, double* part,
-                      cudaStream_t s);
 void launch_cg_dir(int64_t n, const double* sc, const double* z, double* p, cudaStream_t s);
 // Flexible CG (preconditioner applied by the caller between the two):
 // t = r, x += alpha p, r -= alpha q (rr into sc[3]); then with z = M(r),
