@@ -651,7 +651,16 @@ int upload_hierarchy(fs_problem* P, const UnionHierarchy& U, int nc, DHier<T>& D
     std::vector<T> ci(U.dense.begin(), U.dense.end());
     FS_TRY(P->upload(&cinv, ci));
   } else {
-    FS_TRY(invert_on_device<T>(P, U.H.levels.back().A, &cinv));
+    const HostLevel& last = H.levels.back();
+    const int rc = invert_on_device<T>(P, last.A, &cinv);
+    if (rc == FS_ERR_NUMERIC && H.ncoarse <= kHostInverseMax) {
+      std::vector<double> inv;
+      coarse_inverse(last, inv);
+      std::vector<T> ci(inv.begin(), inv.end());
+      FS_TRY(P->upload(&cinv, ci));
+    } else {
+      FS_TRY(rc);
+    }
   }
   D.cinv = cinv;
   int32_t* rb;

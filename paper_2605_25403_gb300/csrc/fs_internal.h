@@ -142,9 +142,17 @@ struct HostLevel {
   int grid[3] = {1, 1, 1};  // structured mesh of the level (cells per axis)
   bool p2 = false;          // the level is the P2 space of that mesh
 };
-// Coarsest operators of at most this many rows are inverted on the host at
-// set-up; larger ones (single problems only) are inverted on the device.
+// Coarsest operators are inverted at set-up: those of a batch's instances on
+// the host (in parallel), a single problem's on the device when it has more
+// than kDeviceInverseMin rows (the host's n^3 against the device's 3 n
+// small launches: one core of an x86 host takes 47 ms at 625 rows and 8 ms at
+// 361; a server of ten mixed requests, which sets up a problem each, went
+// from 305 to 185 ms with the line at 320 rather than 800 rows and the host's
+// elimination in place).  Up to
+// kHostInverseMax rows an operator that the device finds singular goes to
+// the host, which falls back to its Jacobi inverse.
 constexpr int64_t kHostInverseMax = 800;
+constexpr int64_t kDeviceInverseMin = 320;
 
 struct HostHierarchy {
   std::vector<HostLevel> levels;   // levels[0] finest; last = coarsest
@@ -158,9 +166,13 @@ struct HostHierarchy {
 // n0 (cells per axis) of the P1 levels, whether level 0 is the P2 space of
 // that mesh (then the first prolongation is P1 -> P2 on the same mesh), and
 // the fine rows whose prolongation rows are zeroed (fixed values).
+// device_inverse: coarse_inv is left empty above kDeviceInverseMin rows.
 void build_hierarchy(const Mesh& m, const HostCsr& A0, bool p2_fine,
                      const std::vector<int32_t>& fixed_rows,
-                     int64_t coarse_max, HostHierarchy& H);
+                     int64_t coarse_max, HostHierarchy& H, bool device_inverse);
+// Dense inverse of a level's operator on the host, its Jacobi inverse when it
+// is singular.
+void coarse_inverse(const HostLevel& L, std::vector<double>& inv);
 
 // Hierarchy of a batched (union) mesh: one hierarchy per instance (built in
 // parallel), combined level by level into block-diagonal operators.  An
@@ -177,7 +189,7 @@ struct UnionHierarchy {
   std::vector<double> dense;         // concatenated dense inverses (row-major);
                                      // empty: invert the coarsest level's A
                                      // on the device (one block above
-                                     // kHostInverseMax rows)
+                                     // kDeviceInverseMin rows)
   std::vector<int32_t> row_blk;      // coarsest row -> instance
   // per level: first row of each instance (instance count + 1 entries;
   // every level is block-diagonal in instance order)
