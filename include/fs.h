@@ -456,10 +456,13 @@ typedef struct {
   int64_t tail_rows_velocity;
   int64_t tail_rows_pressure;
   int32_t spmv_group;    /* SELL slots a thread issues together in the SpMV:
-                            4, 6 or 8; 0 = 6 in FP32, 4 in FP64 */
+                            4, 6 or 8; 0 = 6 in FP32, 4 in FP64, and on
+                            small problems (FP64, or 3D) 4 or 8 warps
+                            share the rows of a slice                  */
   int32_t smooth_group;  /* ... in the smoothing passes: 4 or 6; 0 = 8 in
                             FP32, 4 in FP64 (8 on levels of at most 8
-                            entries a row)                              */
+                            entries a row), and rows shared by 4 or 8
+                            warps on small levels (FP64, or 3D)         */
   int32_t coarse_degree; /* degree of the Chebyshev smoother on the levels
                             below the finest (pre and post): 3, 2 or 1;
                             0 = 2 (1: the first step of the restriction is

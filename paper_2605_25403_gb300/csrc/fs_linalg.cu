@@ -66,6 +66,150 @@ __device__ __forceinline__ constexpr bool skip_padding() {
 // x 3 values in 3D), the longest work per thread, and the blocks scheduled
 // first start first instead of forming a tail.
 // ---------------------------------------------------------------------------
+// ---------------------------------------------------------------------------
+// Warps per slice of 32 rows.
+//
+// A thread per row leaves most of the chip idle on small problems, and a
+// row's chain of loads (offset, columns, gathers; 65 slots in eight or more
+// groups in 3D) and, in FP64, its FMAs (64 cycles of a quarter SM per warp)
+// are then the kernel's whole time.  Below the sizes here a block takes one
+// slice and its 4 or 8 warps a share of every row's slots; a barrier and the
+// sum of the shares cost about 0.5 us and, once the chip is full, time of
+// their own, so the thread-per-row kernels stay above them.  Measured, us
+// before -> after for one application of the preconditioner / the
+// saddle-point product, and at the first size past the line with it crossed:
+//   FP32 3D  12^3 66.9 -> 52.2 / 7.9 -> 4.2;  28^3 95.5 -> 103.7, 20^3 8.5 -> 10.3
+//   FP64 2D  64^2 73.6 -> 57.7 / 6.8 -> 4.2;  192^2 142.7 -> 144.9 / 14.7 -> 16.9
+//   FP64 3D  16^3 175 -> 107 / 24.0 -> 13.1;  32^3 362 -> 367, 28^3 51.2 -> 53.1
+// Eight warps against four: 8^3 30.5 -> 29.2 (FP32), 62.2 -> 53.9 (FP64);
+// 12^3 54.1 -> 54.8 and 94.4 -> 88.5; 16^3 58.9 -> 64.0 and 107 -> 109.
+// FP32 rows of 2D meshes (at most 19 slots) are three groups of 8 or fewer
+// and have little to share (64^2 43.1 -> 41.6, 32^2 40.4 -> 41.1 on its
+// narrow levels): they keep a thread per row and its order of summation.
+// ---------------------------------------------------------------------------
+// smoothing passes: bytes of a value, components, rows of the level, slots of
+// its rows (0: they differ)
+constexpr int share_mg(size_t bytes, int nc, int64_t rows, int64_t width) {
+  if (bytes == 4 && nc != 3 && width <= 10) return 1;
+  if (rows > (bytes == 4 ? 120000 : nc == 3 ? 200000 : 80000)) return 1;
+  return rows <= (bytes == 4 ? 8192 : 16384) ? 8 : 4;
+}
+// saddle-point product: bytes of a vector entry, dimension, velocity nodes
+constexpr int share_spmv(size_t bytes, int dim, int64_t n2) {
+  if (bytes == 4 && dim == 2) return 1;
+  if (n2 > (bytes == 4 ? 40000 : dim == 3 ? 120000 : 80000)) return 1;
+  return bytes == 8 && n2 <= 6000 ? 8 : 4;
+}
+// velocity right-hand side of the preconditioner (up to 8 slots in 2D, 18 in
+// 3D; at the lines the two forms are within 1%): FP32 7^3 cube 26.6 -> 24.4
+// us for the preconditioner, FP64 50.2 -> 44.8
+constexpr int share_bt(size_t bytes, int dim, int64_t n2) {
+  if (bytes == 4 && dim == 2) return 1;
+  return n2 <= (bytes == 4 ? 70000 : dim == 3 ? 50000 : 20000) ? 4 : 1;
+}
+
+// The slots of one share of a row: all of them (parts = 1), or the part-th of
+// `parts` runs of consecutive slots.
+__device__ __forceinline__ void slot_share(int w, int part, int parts, int& lo, int& hi) {
+  const int n = (w + parts - 1) / parts;
+  lo = parts == 1 ? 0 : min(part * n, w);
+  hi = parts == 1 ? w : min(lo + n, w);
+}
+
+// acc += (A u - BT p) over one share of a velocity row's slots.
+template <typename T, typename V, int DIM, int kUS>
+__device__ __forceinline__ void spmv_velocity(const DOp<T>& op, const V* __restrict__ x,
+                                              int64_t row, int part, int parts, V (&acc)[DIM]) {
+  const int64_t n2 = op.n2;
+  const V* __restrict__ xp = x + DIM * n2;
+  {
+    const SellRow<T> R(op.A, row);
+    int lo, hi;
+    slot_share(R.w, part, parts, lo, hi);
+    R.with_columns(op.A, [&](auto col, int shift) {
+      const T* __restrict__ v = op.A.v + R.first + R.t;
+      const V* __restrict__ xs = x + shift;
+      for (int k = lo; k < hi; k += kUS) {
+        V a[kUS], g[kUS][DIM];
+#pragma unroll
+        for (int u = 0; u < kUS; ++u) {
+          const bool ok = k + u < hi;
+          a[u] = ok ? (V)v[32 * (k + u)] : V(0);
+          const int32_t j = ok ? col(k + u) : (int32_t)row - shift;
+#pragma unroll
+          for (int c = 0; c < DIM; ++c) g[u][c] = xs[c * n2 + j];
+        }
+#pragma unroll
+        for (int u = 0; u < kUS; ++u) {
+          if (skip_padding<V>() && k + u >= hi) break;
+#pragma unroll
+          for (int c = 0; c < DIM; ++c) acc[c] += a[u] * g[u][c];
+        }
+      }
+    });
+  }
+  // d values per slot, component-major: component c of slot u at
+  // (slice offset + 32 u) d + 32 c + t
+  const SellRow<T> R(op.BT, row);
+  int lo, hi;
+  slot_share(R.w, part, parts, lo, hi);
+  R.with_columns(op.BT, [&](auto col, int shift) {
+    const T* __restrict__ v = op.BT.v + R.first * DIM + R.t;
+    const V* __restrict__ ps = xp + shift;
+    for (int k = lo; k < hi; k += kU) {
+      V p[kU], bv[kU][DIM];
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const bool ok = k + u < hi;
+        p[u] = ok ? ps[col(k + u)] : V(0);
+#pragma unroll
+        for (int c = 0; c < DIM; ++c) bv[u][c] = ok ? (V)v[32 * ((k + u) * DIM + c)] : V(0);
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        if (skip_padding<V>() && k + u >= hi) break;
+#pragma unroll
+        for (int c = 0; c < DIM; ++c) acc[c] -= bv[u][c] * p[u];
+      }
+    }
+  });
+}
+
+// (B u) over one share of a pressure row's slots.
+template <typename T, typename V, int DIM, int kUS>
+__device__ __forceinline__ V spmv_pressure(const DOp<T>& op, const V* __restrict__ x, int64_t q,
+                                           int part, int parts) {
+  const int64_t n2 = op.n2;
+  V acc = V(0);
+  const SellRow<T> R(op.B, q);
+  int lo, hi;
+  slot_share(R.w, part, parts, lo, hi);
+  R.with_columns(op.B, [&](auto col, int shift) {
+    const T* __restrict__ v = op.B.v + R.first * DIM + R.t;
+    const V* __restrict__ xs = x + shift;
+    for (int k = lo; k < hi; k += kUS) {
+      V bv[kUS][DIM], g[kUS][DIM];
+#pragma unroll
+      for (int u = 0; u < kUS; ++u) {
+        const bool ok = k + u < hi;
+        const int32_t j = ok ? col(k + u) : -shift;
+#pragma unroll
+        for (int c = 0; c < DIM; ++c) {
+          bv[u][c] = ok ? (V)v[32 * ((k + u) * DIM + c)] : V(0);
+          g[u][c] = ok ? xs[c * n2 + j] : V(0);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kUS; ++u) {
+        if (skip_padding<V>() && k + u >= hi) break;
+#pragma unroll
+        for (int c = 0; c < DIM; ++c) acc += bv[u][c] * g[u][c];
+      }
+    }
+  });
+  return acc;
+}
+
 template <typename T, typename V, int DIM, int kUS>
 __global__ void __launch_bounds__(256) k_spmv_full(DOp<T> op, JVec<const V> xv,
                                                    const V* __restrict__ b, JVec<V> yv,
@@ -77,62 +221,13 @@ __global__ void __launch_bounds__(256) k_spmv_full(DOp<T> op, JVec<const V> xv,
   V* __restrict__ y = yv.get();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t n2 = op.n2, nv = op.nv, wp = (nv + 31) & ~(int64_t)31;
-  const V* __restrict__ xp = x + DIM * n2;
   if (t >= wp) {
     const int64_t row = t - wp;
     if (row >= n2 || seg_skipped(sku, row)) return;
     V acc[DIM];
 #pragma unroll
     for (int c = 0; c < DIM; ++c) acc[c] = V(0);
-    {
-      const SellRow<T> R(op.A, row);
-      R.with_columns(op.A, [&](auto col, int shift) {
-        const T* __restrict__ v = op.A.v + R.first + R.t;
-        const V* __restrict__ xs = x + shift;
-        for (int k = 0; k < R.w; k += kUS) {
-          V a[kUS], g[kUS][DIM];
-#pragma unroll
-          for (int u = 0; u < kUS; ++u) {
-            const bool ok = k + u < R.w;
-            a[u] = ok ? (V)v[32 * (k + u)] : V(0);
-            const int32_t j = ok ? col(k + u) : (int32_t)row - shift;
-#pragma unroll
-            for (int c = 0; c < DIM; ++c) g[u][c] = xs[c * n2 + j];
-          }
-#pragma unroll
-          for (int u = 0; u < kUS; ++u) {
-            if (skip_padding<V>() && k + u >= R.w) break;
-#pragma unroll
-            for (int c = 0; c < DIM; ++c) acc[c] += a[u] * g[u][c];
-          }
-        }
-      });
-    }
-    {
-      // d values per slot, component-major: component c of slot u at
-      // (slice offset + 32 u) d + 32 c + t
-      const SellRow<T> R(op.BT, row);
-      R.with_columns(op.BT, [&](auto col, int shift) {
-        const T* __restrict__ v = op.BT.v + R.first * DIM + R.t;
-        const V* __restrict__ ps = xp + shift;
-        for (int k = 0; k < R.w; k += kU) {
-          V p[kU], bv[kU][DIM];
-#pragma unroll
-          for (int u = 0; u < kU; ++u) {
-            const bool ok = k + u < R.w;
-            p[u] = ok ? ps[col(k + u)] : V(0);
-#pragma unroll
-            for (int c = 0; c < DIM; ++c) bv[u][c] = ok ? (V)v[32 * ((k + u) * DIM + c)] : V(0);
-          }
-#pragma unroll
-          for (int u = 0; u < kU; ++u) {
-            if (skip_padding<V>() && k + u >= R.w) break;
-#pragma unroll
-            for (int c = 0; c < DIM; ++c) acc[c] -= bv[u][c] * p[u];
-          }
-        }
-      });
-    }
+    spmv_velocity<T, V, DIM, kUS>(op, x, row, 0, 1, acc);
 #pragma unroll
     for (int c = 0; c < DIM; ++c) {
       const int64_t r = c * n2 + row;
@@ -141,35 +236,59 @@ __global__ void __launch_bounds__(256) k_spmv_full(DOp<T> op, JVec<const V> xv,
   } else {
     const int64_t q = t;
     if (q >= nv || seg_skipped(skp, q)) return;
-    V acc = V(0);
-    const SellRow<T> R(op.B, q);
-    R.with_columns(op.B, [&](auto col, int shift) {
-      const T* __restrict__ v = op.B.v + R.first * DIM + R.t;
-      const V* __restrict__ xs = x + shift;
-      for (int k = 0; k < R.w; k += kUS) {
-        V bv[kUS][DIM], g[kUS][DIM];
-#pragma unroll
-        for (int u = 0; u < kUS; ++u) {
-          const bool ok = k + u < R.w;
-          const int32_t j = ok ? col(k + u) : -shift;
-#pragma unroll
-          for (int c = 0; c < DIM; ++c) {
-            bv[u][c] = ok ? (V)v[32 * ((k + u) * DIM + c)] : V(0);
-            g[u][c] = ok ? xs[c * n2 + j] : V(0);
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < kUS; ++u) {
-          if (skip_padding<V>() && k + u >= R.w) break;
-#pragma unroll
-          for (int c = 0; c < DIM; ++c) acc += bv[u][c] * g[u][c];
-        }
-      }
-    });
-    const V v = acc + (V)op.diagp[q] * xp[q];
+    const V acc = spmv_pressure<T, V, DIM, kUS>(op, x, q, 0, 1);
     const int64_t r = DIM * n2 + q;
+    const V v = acc + (V)op.diagp[q] * x[r];
     y[r] = resid ? b[r] - v : v;
   }
+}
+
+// The same with a block per slice of 32 rows, whose W warps take a share of
+// the slots each (pressure slices first); a warp per component adds the
+// shares and finishes the rows.
+template <typename T, typename V, int DIM, int W, int kUS>
+__global__ void __launch_bounds__(32 * W) k_spmv_split(DOp<T> op, JVec<const V> xv,
+                                                       const V* __restrict__ b, JVec<V> yv,
+                                                       int resid, SegSkip sku, SegSkip skp,
+                                                       const int* skip) {
+  static_assert(W >= DIM, "a warp per component");
+  pdl_wait();
+  if (skip && *skip) return;
+  __shared__ V share[W][DIM][32];
+  const V* __restrict__ x = xv.get();
+  V* __restrict__ y = yv.get();
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t n2 = op.n2, nv = op.nv, ps = (nv + 31) >> 5;
+  const bool pres = blockIdx.x < ps;
+  const int64_t row = (pres ? (int64_t)blockIdx.x : blockIdx.x - ps) * 32 + lane;
+  const bool act = pres ? row < nv && !seg_skipped(skp, row) : row < n2 && !seg_skipped(sku, row);
+  V acc[DIM];
+#pragma unroll
+  for (int c = 0; c < DIM; ++c) acc[c] = V(0);
+  if (act) {
+    if (pres) acc[0] = spmv_pressure<T, V, DIM, kUS>(op, x, row, w, W);
+    else spmv_velocity<T, V, DIM, kUS>(op, x, row, w, W, acc);
+  }
+  // the finishing warps' own operands, before the shares are awaited
+  const bool fin = act && w < (pres ? 1 : DIM);
+  const int64_t r = (pres ? DIM : w) * n2 + row;
+  V own = V(0), dq = V(0), xq = V(0);
+  if (fin) {
+    if (resid) own = b[r];
+    if (pres) {
+      dq = (V)op.diagp[row];
+      xq = x[r];
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < DIM; ++c) share[w][c][lane] = acc[c];
+  __syncthreads();
+  if (!fin) return;
+  V v = share[0][w][lane];
+#pragma unroll
+  for (int i = 1; i < W; ++i) v += share[i][w][lane];
+  if (pres) v += dq * xq;
+  y[r] = resid ? own - v : v;
 }
 
 // CSR -> SELL-32 value scatter, one thread per row: the row's entries and its
@@ -257,15 +376,15 @@ __device__ __forceinline__ void vstore(T* __restrict__ p, const T (&v)[N]) {
   }
 }
 
-// acc += (A x) of one row, x row-major with NCP components.  G slots at a
-// time, their loads before their FMAs; the slot count is the same for the
-// whole slice.  Slots past the last one repeat it with coefficient 0, so that
+// acc += (A x) of one row's slots lo .. w, x row-major with NCP components.
+// G slots at a time, their loads before their FMAs; the slot count is the
+// same for the whole slice.  Slots past the last one repeat it with coefficient 0, so that
 // the loads of a partial group are as independent as those of a full one
 // (a branch per slot there chained each column load to its gather).
 template <typename T, int NC, int NCP, int G, typename Col>
-__device__ __forceinline__ void sell_slots(const T* __restrict__ v, int w, Col col,
+__device__ __forceinline__ void sell_slots(const T* __restrict__ v, int lo, int w, Col col,
                                            const T* __restrict__ x, T (&acc)[NCP]) {
-  for (int k = 0; k < w; k += G) {
+  for (int k = lo; k < w; k += G) {
     T a[G], g[G][NCP];
     int32_t j[G];
 #pragma unroll
@@ -285,14 +404,36 @@ __device__ __forceinline__ void sell_slots(const T* __restrict__ v, int w, Col c
 
 template <typename T, int NC, int NCP, int G>
 __device__ __forceinline__ void sell_row_times(const DSell<T>& A, const T* __restrict__ x,
-                                               int64_t row, T (&acc)[NCP]) {
+                                               int64_t row, T (&acc)[NCP], int part = 0,
+                                               int parts = 1) {
   const SellRow<T> R(A, row);
   const T* __restrict__ v = A.v + R.first + R.t;
+  int lo, hi;
+  slot_share(R.w, part, parts, lo, hi);
 #pragma unroll
   for (int c = 0; c < NCP; ++c) acc[c] = T(0);
   R.with_columns(A, [&](auto col, int shift) {
-    sell_slots<T, NC, NCP, G>(v, R.w, col, x + shift * NCP, acc);
+    sell_slots<T, NC, NCP, G>(v, lo, hi, col, x + shift * NCP, acc);
   });
+}
+
+// One component of a row's Chebyshev pass from acc = (A Gin) of the row, the
+// row's own gx = Gin, d = Din and right-hand side bb.
+template <typename T, int MODE>
+__device__ __forceinline__ void mg_component(T acc, T di, T bb, T gx, T d, T alpha, T beta,
+                                             T inv_theta, T& go, T& dout) {
+  const T r = bb - acc;
+  if (MODE == MG_STEP) {
+    dout = alpha * d + beta * di * r;
+    go = gx + dout;
+  } else if (MODE == MG_RESID) {
+    go = r;
+  } else if (MODE == MG_START) {
+    dout = di * r * inv_theta;
+    go = gx + dout;
+  } else {
+    go = gx + (alpha * d + beta * di * r);
+  }
 }
 
 // The row's own part of a Chebyshev pass: acc = (A Gin) of the row.
@@ -303,7 +444,7 @@ __device__ __forceinline__ void mg_finish(const T (&acc)[NCP], const T* __restri
                                           T* __restrict__ Dout, T alpha, T beta, T inv_theta,
                                           T* __restrict__ out, int64_t out_ld,
                                           const int32_t* __restrict__ perm, int nc, int64_t row) {
-  T gx[NCP], d[NCP], bb[NCP];
+  T gx[NCP], d[NCP] = {}, bb[NCP];
   vload<T, NCP>(Gin + row * NCP, gx);
   if (MODE == MG_STEP || MODE == MG_LAST) vload<T, NCP>(Din + row * NCP, d);
   vload<T, NCP>(b + row * NCP, bb);
@@ -315,20 +456,8 @@ __device__ __forceinline__ void mg_finish(const T (&acc)[NCP], const T* __restri
     dout[c] = T(0);
   }
 #pragma unroll
-  for (int c = 0; c < NC; ++c) {
-    const T r = bb[c] - acc[c];
-    if (MODE == MG_STEP) {
-      dout[c] = alpha * d[c] + beta * di * r;
-      go[c] = gx[c] + dout[c];
-    } else if (MODE == MG_RESID) {
-      go[c] = r;
-    } else if (MODE == MG_START) {
-      dout[c] = di * r * inv_theta;
-      go[c] = gx[c] + dout[c];
-    } else {
-      go[c] = gx[c] + (alpha * d[c] + beta * di * r);
-    }
-  }
+  for (int c = 0; c < NC; ++c)
+    mg_component<T, MODE>(acc[c], di, bb[c], gx[c], d[c], alpha, beta, inv_theta, go[c], dout[c]);
   if (MODE == MG_LAST && out) {
     const int64_t dst = perm ? perm[row] : row;
     for (int c = 0; c < nc; ++c) out[c * out_ld + dst] = go[c];
@@ -515,6 +644,59 @@ __global__ void __launch_bounds__(256) k_mg(DSell<T> A, const T* __restrict__ di
   if (row >= A.nrow || seg_skipped(sk, row)) return;
   mg_row<T, NC, NCP, MODE, G>(A, dinv, b, Gin, Din, Gout, Dout, alpha, beta, inv_theta,
                                   MODE == MG_LAST ? outv.get() : nullptr, out_ld, perm, nc, row);
+}
+
+// The same with a block per slice of 32 rows, whose W warps take a share of
+// the slots each; a warp per component adds the shares and finishes the rows.
+template <typename T, int NC, int NCP, int MODE, int W, int G>
+__global__ void __launch_bounds__(32 * W) k_mg_split(DSell<T> A, const T* __restrict__ dinv,
+                                                     const T* __restrict__ b,
+                                                     const T* __restrict__ Gin,
+                                                     const T* __restrict__ Din,
+                                                     T* __restrict__ Gout, T* __restrict__ Dout,
+                                                     T alpha, T beta, T inv_theta, JVec<T> outv,
+                                                     int64_t out_ld,
+                                                     const int32_t* __restrict__ perm, int nc,
+                                                     SegSkip sk, const int* skip) {
+  static_assert(W >= NCP, "a warp per component");
+  pdl_wait();
+  if (skip && *skip) return;
+  __shared__ T share[W][NC][32];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t row = blockIdx.x * (int64_t)32 + lane;
+  const bool act = row < A.nrow && !seg_skipped(sk, row);
+  T acc[NCP] = {};
+  if (act) sell_row_times<T, NC, NCP, G>(A, Gin, row, acc, w, W);
+  // the finishing warps' own operands, before the shares are awaited
+  const bool fin = act && w < NCP;
+  const int64_t e = row * NCP + w;
+  T* __restrict__ out = MODE == MG_LAST ? outv.get() : nullptr;
+  T gx = T(0), d = T(0), bb = T(0), di = T(0);
+  int64_t dst = row;
+  if (fin && w < NC) {
+    gx = Gin[e];
+    if (MODE == MG_STEP || MODE == MG_LAST) d = Din[e];
+    bb = b[e];
+    di = dinv[row];
+    if (out && perm) dst = perm[row];
+  }
+#pragma unroll
+  for (int c = 0; c < NC; ++c) share[w][c][lane] = acc[c];
+  __syncthreads();
+  if (!fin) return;
+  T go = T(0), dout = T(0);
+  if (w < NC) {
+    T a = share[0][w][lane];
+#pragma unroll
+    for (int i = 1; i < W; ++i) a += share[i][w][lane];
+    mg_component<T, MODE>(a, di, bb, gx, d, alpha, beta, inv_theta, go, dout);
+  }
+  if (MODE == MG_LAST && out) {
+    if (w < nc) out[w * out_ld + dst] = go;
+    return;
+  }
+  Gout[e] = go;
+  if (MODE == MG_STEP || MODE == MG_START) Dout[e] = dout;
 }
 
 template <typename T, int NCP, int L>
@@ -748,20 +930,28 @@ void launch_mg(int mode, const DLevel<T>& L, const T* b, const T* Gin, const T* 
   constexpr bool f32 = std::is_same<T, float>::value;
   const int g = group ? group : f32 || (L.A.width > 0 && L.A.width <= 8) ? 8 : 4;
   constexpr int kB = f32 ? 256 : 128;
+  const int share = group ? 1 : share_mg(sizeof(T), NC, n, L.A.width);
+#define FS_MGS(M, W)                                                                           \
+  launch_k(k_mg_split<T, NC, NCP, M, W, f32 ? 8 : 4>, (unsigned)((n + 31) / 32), 32 * W, 0, s, \
+           L.A, L.dinv, b, Gin, Din, Gout, Dout, alpha, beta, it, out, out_ld, perm, nc, L.skip, \
+           skip)
 #define FS_MG(M, G)                                                                        \
   launch_k(k_mg<T, NC, NCP, M, G>, blocks_for(n, kB), kB, 0, s, L.A, L.dinv, b, Gin, Din, Gout, \
            Dout, alpha, beta, it, out, out_ld, perm, nc, L.skip, skip)
-#define FS_MG_MODES(G)                              \
-  do {                                              \
-    if (mode == MG_STEP) FS_MG(MG_STEP, G);         \
-    else if (mode == MG_RESID) FS_MG(MG_RESID, G);  \
-    else if (mode == MG_START) FS_MG(MG_START, G);  \
-    else FS_MG(MG_LAST, G);                         \
+#define FS_MG_MODES(F, G)                      \
+  do {                                         \
+    if (mode == MG_STEP) F(MG_STEP, G);        \
+    else if (mode == MG_RESID) F(MG_RESID, G); \
+    else if (mode == MG_START) F(MG_START, G); \
+    else F(MG_LAST, G);                        \
   } while (0)
-  if (g == 8) FS_MG_MODES(8);
-  else if (g == 6) FS_MG_MODES(6);
-  else FS_MG_MODES(4);
+  if (share == 8) FS_MG_MODES(FS_MGS, 8);
+  else if (share == 4) FS_MG_MODES(FS_MGS, 4);
+  else if (g == 8) FS_MG_MODES(FS_MG, 8);
+  else if (g == 6) FS_MG_MODES(FS_MG, 6);
+  else FS_MG_MODES(FS_MG, 4);
 #undef FS_MG_MODES
+#undef FS_MGS
 #undef FS_MG
   count_launches(1);
 }
@@ -803,7 +993,11 @@ void vcycle_level(const DHier<T>& H, int l, JVec<T> out, int64_t out_ld, int nc,
     return;
   }
   if (l == H.nlev - 1) {
-    launch_k(k_mg_dense<T, NCP>, blocks_for(H.ncoarse * 32), 256, 0, s,
+    // FP64: few warps per SM quarter, whose FMAs and sums are its time
+    // (289 rows 11.6 -> 10.8 us for the V-cycle of the 8^2 square; larger
+    // blocks and FP32 within 1%)
+    constexpr unsigned db = std::is_same<T, double>::value ? 128 : 256;
+    launch_k(k_mg_dense<T, NCP>, blocks_for(H.ncoarse * 32, db), db, 0, s,
         dense_view(H), H.ncoarse, H.b[l], H.G1[l], top ? H.perm : nullptr,
         top ? out : JVec<T>(), out_ld, nc, H.lev[l].skip, skip);
     count_launches(1);
@@ -1005,44 +1199,24 @@ __device__ __forceinline__ T cc_combine(const T* __restrict__ mpl, const T* __re
   return m < T(0) ? p : m * p + inv_dt * yk[q];
 }
 
-template <typename T, int DIM, int NCP, bool ZREAD>
-__global__ void __launch_bounds__(256) k_bt_add_mg(DSell<T> BT, int64_t n2, int64_t nv,
-                                                   JVec<const T> rv, const T* __restrict__ yk,
-                                                   const T* __restrict__ mpl, T inv_dt,
-                                                   JVec<T> zv, const int32_t* __restrict__ iperm,
-                                                   const T* __restrict__ dinv0, T inv_theta0,
-                                                   T* __restrict__ b0, T* __restrict__ G0,
-                                                   T* __restrict__ D0, SegSkip sk0,
-                                                   const int* skip) {
-  pdl_wait();
-  if (skip && *skip) return;
-  const T* __restrict__ r = rv.get();
-  const T* __restrict__ rp = r + DIM * n2;
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t nvp = (nv + 31) & ~(int64_t)31;
-  // ZREAD: z_p was written by the pressure kernel before (convection-
-  // diffusion form), read it back
-  const T* __restrict__ zp = zv.get() + DIM * n2;
-  if (t < nvp) {
-    if (!ZREAD && t < nv) zv.get()[DIM * n2 + t] = cc_combine(mpl, rp, yk, inv_dt, t);
-    return;
-  }
-  const int64_t row = t - nvp;
-  if (row >= n2) return;
-  const int64_t dst = iperm ? iperm[row] : row;
-  if (seg_skipped(sk0, dst)) return;
-  T acc[DIM];
-#pragma unroll
-  for (int c = 0; c < DIM; ++c) acc[c] = T(0);
+// acc += (BT z_p) over one share of a velocity row's slots (ZREAD: z_p was
+// written by the pressure kernel before, read it back).
+template <typename T, int DIM, bool ZREAD>
+__device__ __forceinline__ void bt_slots(const DSell<T>& BT, int64_t row, int part, int parts,
+                                         const T* zp, const T* __restrict__ mpl,
+                                         const T* __restrict__ rp, const T* __restrict__ yk,
+                                         T inv_dt, T (&acc)[DIM]) {
   const SellRow<T> R(BT, row);
+  int lo, hi;
+  slot_share(R.w, part, parts, lo, hi);
   R.with_columns(BT, [&](auto col, int shift) {
     const T* __restrict__ v = BT.v + R.first * DIM + R.t;
-    for (int k = 0; k < R.w; k += kU) {
+    for (int k = lo; k < hi; k += kU) {
       T p[kU], bv[kU][DIM];
 #pragma unroll
       for (int u = 0; u < kU; ++u) {
         p[u] = T(0);
-        if (k + u < R.w) {
+        if (k + u < hi) {
           const int32_t j = col(k + u) + shift;
           p[u] = ZREAD ? zp[j] : cc_combine(mpl, rp, yk, inv_dt, j);
 #pragma unroll
@@ -1058,6 +1232,36 @@ __global__ void __launch_bounds__(256) k_bt_add_mg(DSell<T> BT, int64_t n2, int6
         for (int c = 0; c < DIM; ++c) acc[c] += bv[u][c] * p[u];
     }
   });
+}
+
+template <typename T, int DIM, int NCP, bool ZREAD>
+__global__ void __launch_bounds__(256) k_bt_add_mg(DSell<T> BT, int64_t n2, int64_t nv,
+                                                   JVec<const T> rv, const T* __restrict__ yk,
+                                                   const T* __restrict__ mpl, T inv_dt,
+                                                   JVec<T> zv, const int32_t* __restrict__ iperm,
+                                                   const T* __restrict__ dinv0, T inv_theta0,
+                                                   T* __restrict__ b0, T* __restrict__ G0,
+                                                   T* __restrict__ D0, SegSkip sk0,
+                                                   const int* skip) {
+  pdl_wait();
+  if (skip && *skip) return;
+  const T* __restrict__ r = rv.get();
+  const T* __restrict__ rp = r + DIM * n2;
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t nvp = (nv + 31) & ~(int64_t)31;
+  const T* zp = zv.get() + DIM * n2;
+  if (t < nvp) {
+    if (!ZREAD && t < nv) zv.get()[DIM * n2 + t] = cc_combine(mpl, rp, yk, inv_dt, t);
+    return;
+  }
+  const int64_t row = t - nvp;
+  if (row >= n2) return;
+  const int64_t dst = iperm ? iperm[row] : row;
+  if (seg_skipped(sk0, dst)) return;
+  T acc[DIM];
+#pragma unroll
+  for (int c = 0; c < DIM; ++c) acc[c] = T(0);
+  bt_slots<T, DIM, ZREAD>(BT, row, 0, 1, zp, mpl, rp, yk, inv_dt, acc);
   T tv[NCP], d0[NCP];
   const T sc = dinv0 ? dinv0[dst] * inv_theta0 : T(0);
 #pragma unroll
@@ -1068,6 +1272,59 @@ __global__ void __launch_bounds__(256) k_bt_add_mg(DSell<T> BT, int64_t n2, int6
   vstore<T, NCP>(b0 + dst * NCP, tv);
   vstore<T, NCP>(G0 + dst * NCP, d0);
   vstore<T, NCP>(D0 + dst * NCP, d0);
+}
+
+// The same with a block per 32 velocity rows, whose W warps take a share of
+// the slots each; a warp per component adds the shares and finishes the rows.
+template <typename T, int DIM, int NCP, bool ZREAD, int W>
+__global__ void __launch_bounds__(32 * W) k_bt_add_split(
+    DSell<T> BT, int64_t n2, int64_t nv, JVec<const T> rv, const T* __restrict__ yk,
+    const T* __restrict__ mpl, T inv_dt, JVec<T> zv, const int32_t* __restrict__ iperm,
+    const T* __restrict__ dinv0, T inv_theta0, T* __restrict__ b0, T* __restrict__ G0,
+    T* __restrict__ D0, SegSkip sk0, const int* skip) {
+  static_assert(W >= NCP, "a warp per component");
+  pdl_wait();
+  if (skip && *skip) return;
+  __shared__ T share[W][DIM][32];
+  const T* __restrict__ r = rv.get();
+  const T* __restrict__ rp = r + DIM * n2;
+  T* zp = zv.get() + DIM * n2;
+  const int64_t pb = (nv + 32 * W - 1) / (32 * W);  // blocks of pressure rows
+  if (blockIdx.x < pb) {
+    const int64_t q = blockIdx.x * (int64_t)(32 * W) + threadIdx.x;
+    if (!ZREAD && q < nv) zp[q] = cc_combine(mpl, rp, yk, inv_dt, q);
+    return;
+  }
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t row = (blockIdx.x - pb) * 32 + lane;
+  int64_t dst = row;
+  bool act = row < n2;
+  if (act) {
+    if (iperm) dst = iperm[row];
+    act = !seg_skipped(sk0, dst);
+  }
+  T acc[DIM] = {};
+  if (act) bt_slots<T, DIM, ZREAD>(BT, row, w, W, zp, mpl, rp, yk, inv_dt, acc);
+  const bool fin = act && w < NCP;
+  T sc = T(0), tv = T(0);
+  if (fin && w < DIM) {
+    sc = dinv0 ? dinv0[dst] * inv_theta0 : T(0);
+    tv = r[w * n2 + row];
+  }
+#pragma unroll
+  for (int c = 0; c < DIM; ++c) share[w][c][lane] = acc[c];
+  __syncthreads();
+  if (!fin) return;
+  if (w < DIM) {
+    T a = share[0][w][lane];
+#pragma unroll
+    for (int i = 1; i < W; ++i) a += share[i][w][lane];
+    tv += a;
+  }
+  const int64_t e = dst * NCP + w;
+  b0[e] = tv;
+  G0[e] = sc * tv;
+  D0[e] = sc * tv;
 }
 
 // Gauss-Jordan step c on W = [A | I] (n x 2n, row-major).  The pivot is the
@@ -1180,10 +1437,24 @@ void launch_spmv_full(const DOp<T>& op, JVec<const V> x, const V* b, JVec<V> y, 
   // slots per group: the schedule's, else 6 in FP32 and 4 in FP64 (FP64
   // rows are partly bound by FP64 arithmetic and do best shallower)
   const int g = op.group ? op.group : (std::is_same<V, float>::value ? kUSpmv : kU);
+  constexpr bool f32 = std::is_same<V, float>::value;
+  const int share = op.group ? 1 : share_spmv(sizeof(V), op.dim, op.n2);
+#define FS_SPMVS(D, W)                                                                     \
+  launch_k(k_spmv_split<T, V, D, W, f32 ? 8 : 4>,                                          \
+           (unsigned)((op.nv + 31) / 32 + (op.n2 + 31) / 32), 32 * W, 0, s, op, x, b, y, resid, \
+           su, sp, skip)
 #define FS_SPMV(D, G) \
   launch_k(k_spmv_full<T, V, D, G>, blocks_for(threads), 256, 0, s, op, x, b, y, resid, su, sp, \
            skip)
-  if (op.dim == 2) {
+  if (share > 1) {
+    if (op.dim == 2) {
+      if (share == 8) FS_SPMVS(2, 8);
+      else FS_SPMVS(2, 4);
+    } else {
+      if (share == 8) FS_SPMVS(3, 8);
+      else FS_SPMVS(3, 4);
+    }
+  } else if (op.dim == 2) {
     if (g == 8) FS_SPMV(2, 8);
     else if (g == 6) FS_SPMV(2, 6);
     else FS_SPMV(2, 4);
@@ -1192,6 +1463,7 @@ void launch_spmv_full(const DOp<T>& op, JVec<const V> x, const V* b, JVec<V> y, 
     else if (g == 6) FS_SPMV(3, 6);
     else FS_SPMV(3, 4);
   }
+#undef FS_SPMVS
 #undef FS_SPMV
   count_launches(1);
 }
@@ -1274,16 +1546,24 @@ void launch_precond(const DOp<T>& op, const DHier<T>& HA, const DHier<T>& HK,
              (T)inv_dt, pcd, z.shifted(dim * n2), skip);
     count_launches(1);
   }
+  auto bt = [&](auto k, unsigned blocks, unsigned threads) {
+    launch_k(k, blocks, threads, 0, s, op.BT, n2, nv, r, (const T*)work_p, mpl_inv_nu, (T)inv_dt,
+             z, HA.iperm, d0, it0, HA.b[0], HA.G0[0], HA.D0[0], HA.lev[0].skip, skip);
+  };
+  const bool split = share_bt(sizeof(T), dim, n2) > 1;
+  const unsigned ns = (unsigned)((nv + 127) / 128 + (n2 + 31) / 32);
   if (dim == 2) {
-    launch_k(pc ? k_bt_add_mg<T, 2, 2, true> : k_bt_add_mg<T, 2, 2, false>, nb, 256, 0, s,
-             op.BT, n2, nv, r, (const T*)work_p, mpl_inv_nu, (T)inv_dt, z, HA.iperm, d0, it0,
-             HA.b[0], HA.G0[0], HA.D0[0], HA.lev[0].skip, skip);
+    if (split)
+      bt(pc ? k_bt_add_split<T, 2, 2, true, 4> : k_bt_add_split<T, 2, 2, false, 4>, ns, 128);
+    else
+      bt(pc ? k_bt_add_mg<T, 2, 2, true> : k_bt_add_mg<T, 2, 2, false>, nb, 256);
     count_launches(1);
     vcycle_level<T, 2>(HA, 0, z, n2, 2, skip, s);
   } else {
-    launch_k(pc ? k_bt_add_mg<T, 3, 4, true> : k_bt_add_mg<T, 3, 4, false>, nb, 256, 0, s,
-             op.BT, n2, nv, r, (const T*)work_p, mpl_inv_nu, (T)inv_dt, z, HA.iperm, d0, it0,
-             HA.b[0], HA.G0[0], HA.D0[0], HA.lev[0].skip, skip);
+    if (split)
+      bt(pc ? k_bt_add_split<T, 3, 4, true, 4> : k_bt_add_split<T, 3, 4, false, 4>, ns, 128);
+    else
+      bt(pc ? k_bt_add_mg<T, 3, 4, true> : k_bt_add_mg<T, 3, 4, false>, nb, 256);
     count_launches(1);
     vcycle_level<T, 4>(HA, 0, z, n2, 3, skip, s);
   }
