@@ -680,51 +680,73 @@ __global__ void k_exact_state(DMesh m, DPhys ph, double t, int zero_interior,
   }
 }
 
-// Monolithic values in paper order, one internal row per thread.  The
+// A warp's rank of the keys of a row of w entries: body(k, rank) for every
+// entry k of [k0, k0 + w), rank = how many of the row's keys nat[ci[.]] are
+// smaller (they are all different).
+template <typename F>
+__device__ __forceinline__ void ranked_row(const int32_t* __restrict__ nat,
+                                           const int32_t* __restrict__ ci, int32_t k0, int32_t w,
+                                           int lane, F body) {
+  for (int32_t b = 0; b < w; b += 32) {
+    const bool in = b + lane < w;
+    const int32_t key = in ? nat[ci[k0 + b + lane]] : 0;
+    int rank = 0;
+    for (int32_t b2 = 0; b2 < w; b2 += 32) {
+      const int32_t other =
+          b2 == b ? key : b2 + lane < w ? nat[ci[k0 + b2 + lane]] : 0;
+      const int n = w - b2 < 32 ? w - b2 : 32;
+      for (int t = 0; t < n; ++t) rank += __shfl_sync(0xffffffffu, other, t) < key;
+    }
+    if (in) body(k0 + b + lane, rank);
+  }
+}
+
+// Monolithic values in paper order, a warp per internal row.  The
 // paper-order row of internal velocity row (c, q) is c n2 + nat[q]; its
 // columns are the row's P2 neighbours in paper order (the rank of nat[j]
 // among the row's entries gives the place), then its pressure neighbours
 // (vertex ids are the same in both orders).  A pressure row keeps its place
 // and holds, per component, its P2 neighbours ranked the same way, then the
 // diagonal.
-__global__ void k_expand_monolithic(DMesh m, const int32_t* __restrict__ nat,
-                                    const double* __restrict__ valA,
-                                    const double* __restrict__ B,
-                                    const double* __restrict__ BT,
-                                    const double* __restrict__ diagp,
-                                    const int64_t* __restrict__ mrp,
-                                    double* __restrict__ out) {
-  const int dim = m.dim;
-  const int64_t nrow = dim * m.n2 + m.nv;
-  for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < nrow;
-       r += (int64_t)gridDim.x * blockDim.x) {
-    if (r < dim * m.n2) {
-      const int c = (int)(r / m.n2);
-      const int64_t i = r % m.n2;
-      int64_t o = mrp[c * m.n2 + nat[i]];
-      const int32_t k0 = m.rpA[i], k1 = m.rpA[i + 1];
-      for (int32_t k = k0; k < k1; ++k) {
-        const int32_t key = nat[m.ciA[k]];
-        int rank = 0;
-        for (int32_t k2 = k0; k2 < k1; ++k2) rank += nat[m.ciA[k2]] < key;
-        out[o + rank] = valA[k];
+//
+// A row's keys are loaded once, by its lanes, and compared by shuffles; the
+// rank serves all components, whose entries a warp writes next to each
+// other.  A thread per row and component, which compared every pair of
+// entries through loads (up to 65^2 per row in 3D) and wrote 8 bytes per
+// row at a time, took most of an export (24^3 cube, assembly and
+// export: 1.47 -> 0.52 ms).
+__global__ void __launch_bounds__(256) k_expand_monolithic(
+    DMesh m, const int32_t* __restrict__ nat, const double* __restrict__ valA,
+    const double* __restrict__ B, const double* __restrict__ BT,
+    const double* __restrict__ diagp, const int64_t* __restrict__ mrp,
+    double* __restrict__ out) {
+  const int dim = m.dim, lane = threadIdx.x & 31;
+  const int64_t n2 = m.n2, nrow = n2 + m.nv, step = (int64_t)gridDim.x * (blockDim.x / 32);
+  for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32; r < nrow; r += step) {
+    if (r < n2) {
+      int64_t o[3] = {0, 0, 0};
+      for (int c = 0; c < dim; ++c) o[c] = mrp[c * n2 + nat[r]];
+      const int32_t k0 = m.rpA[r], w = m.rpA[r + 1] - k0;
+      ranked_row(nat, m.ciA, k0, w, lane, [&](int32_t k, int rank) {
+        const double v = valA[k];
+        out[o[0] + rank] = v;
+        out[o[1] + rank] = v;
+        if (dim == 3) out[o[2] + rank] = v;
+      });
+      const int32_t b0 = m.rpBT[r], b1 = m.rpBT[r + 1];
+      for (int32_t k = b0 + lane; k < b1; k += 32) {
+        const int64_t at = w + (k - b0);
+        out[o[0] + at] = -BT[(int64_t)k * dim];
+        out[o[1] + at] = -BT[(int64_t)k * dim + 1];
+        if (dim == 3) out[o[2] + at] = -BT[(int64_t)k * dim + 2];
       }
-      o += k1 - k0;
-      for (int32_t k = m.rpBT[i]; k < m.rpBT[i + 1]; ++k) out[o++] = -BT[(int64_t)k * dim + c];
     } else {
-      const int64_t q = r - dim * m.n2;
-      int64_t o = mrp[r];
-      const int32_t k0 = m.rpB[q], k1 = m.rpB[q + 1];
-      for (int c = 0; c < dim; ++c) {
-        for (int32_t k = k0; k < k1; ++k) {
-          const int32_t key = nat[m.ciB[k]];
-          int rank = 0;
-          for (int32_t k2 = k0; k2 < k1; ++k2) rank += nat[m.ciB[k2]] < key;
-          out[o + rank] = B[(int64_t)k * dim + c];
-        }
-        o += k1 - k0;
-      }
-      out[o] = diagp[q];
+      const int64_t q = r - n2, o = mrp[dim * n2 + q];
+      const int32_t k0 = m.rpB[q], w = m.rpB[q + 1] - k0;
+      ranked_row(nat, m.ciB, k0, w, lane, [&](int32_t k, int rank) {
+        for (int c = 0; c < dim; ++c) out[o + c * (int64_t)w + rank] = B[(int64_t)k * dim + c];
+      });
+      if (lane == 0) out[o + dim * (int64_t)w] = diagp[q];
     }
   }
 }
@@ -861,8 +883,9 @@ void launch_exact_state(const DMesh& m, const DPhys& ph, double t,
 void launch_expand_monolithic(const DMesh& m, const int32_t* nat, const double* valA,
                               const double* B, const double* BT, const double* diagp,
                               const int64_t* mrp, double* out, cudaStream_t s) {
-  int64_t nrow = m.dim * m.n2 + m.nv;
-  k_expand_monolithic<<<grid_for(nrow, 256), 256, 0, s>>>(m, nat, valA, B, BT, diagp, mrp, out);
+  const int64_t nrow = m.n2 + m.nv;  // a warp each
+  k_expand_monolithic<<<grid_for(nrow * 32, 256), 256, 0, s>>>(m, nat, valA, B, BT, diagp, mrp,
+                                                               out);
   count_launches(1);
 }
 
