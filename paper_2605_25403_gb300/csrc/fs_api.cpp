@@ -1064,8 +1064,8 @@ void issue_check(fs_problem* P, Precision<T>& pr, const T* x, const T* b) {
 // up to m Arnoldi steps, update of x.  Launched directly, the m steps are
 // issued one by one (steps after convergence exit at once).  Captured in a
 // graph, one step is captured as the body of a conditional WHILE node whose
-// condition the device sets (the cycle init, then every step's Givens
-// kernel), so the graph runs exactly the steps the cycle needs.
+// condition the device sets (the cycle init, then the end of every step's
+// orthogonalisation), so the graph runs exactly the steps the cycle needs.
 template <typename T>
 int issue_iter(fs_problem* P, Precision<T>& pr, T* x, int relative_to_beta) {
   Krylov<T>& K = pr.kr;

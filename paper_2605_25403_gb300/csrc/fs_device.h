@@ -600,7 +600,7 @@ void launch_seg_norm(const V* x, const TileList& tl, SegState* st, double* parti
                      int field, cudaStream_t s);
 // cond: the handle of a conditional loop node replaying the Arnoldi step
 // (0 when the steps are launched one by one); the cycle init sets it to
-// "not every segment done", the Givens kernel to "not done and j < m".
+// "not every segment done", the orthogonalisation to "not done and j < m".
 void launch_seg_cycle_init(SegState* st, KCtl* ctl, int relative_to_beta,
                            cudaGraphConditionalHandle cond, cudaStream_t s);
 template <typename V>

@@ -1,5 +1,5 @@
 // Segmented reductions and updates of flexible GMRES(m) (paper Sec. 3.2,
-// GMRES) on sm_103a.
+// GMRES) on sm_103a; fs_orth.cu holds the orthogonalisation.
 //
 // A problem holds one or more independent instances ("segments": the
 // instances of a batch, or the single mesh of an ordinary problem).  Every
@@ -24,9 +24,7 @@ namespace fs {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-// threads per tile block: the orthogonalisation passes stream the basis
-// with few blocks (one per tile), so each block brings many warps, and each
-// thread issues several independent loads, to keep enough bytes in flight
+// threads per tile block: few blocks (one per tile), so each brings many warps
 constexpr int kKB = 512;
 
 template <typename V>
