@@ -975,6 +975,7 @@ int alloc_krylov(fs_problem* P, Krylov<V>& K, int m, const std::vector<int>& fir
   KCtl c{};
   c.m = m;
   c.nseg = P->nseg;
+  c.wait_ns = kWaitNs;
   FS_CUDA(cudaMemcpyAsync(K.ctl, &c, sizeof(KCtl), cudaMemcpyHostToDevice, P->stream));
   FS_CUDA(cudaStreamSynchronize(P->stream));  // host sources go out of scope
   return FS_OK;

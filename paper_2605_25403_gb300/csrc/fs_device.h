@@ -593,7 +593,9 @@ struct KCtl {
   int nredo;     // segments whose orthogonalisation needs a second pass
   unsigned bar, bar_base;  // grid barrier of the orthogonalisation kernel:
                            // arrivals, and their count before the launch
+  uint64_t wait_ns;        // limit of each of that kernel's waits
 };
+constexpr uint64_t kWaitNs = 1000000000ull;  // one second
 
 template <typename V>
 void launch_seg_norm(const V* x, const TileList& tl, SegState* st, double* partial,

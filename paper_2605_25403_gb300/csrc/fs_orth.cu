@@ -63,7 +63,6 @@ constexpr int kOrthMain = 32 * kOrthWarps;       // threads that work on entries
 constexpr int kOneThreads = kOrthMain + 32;      // k_orth_one: and a Givens warp
 constexpr int kManyThreads = kOrthMain + 64;     // k_orth_many: a copying and a Givens warp
 constexpr double kRedo = 0.01;
-constexpr uint64_t kOrthWaitNs = 1000000000ull;  // one second per wait
 static_assert(kMaxRestart <= 32, "a lane per basis vector");
 
 template <typename V>
@@ -93,13 +92,14 @@ __device__ __forceinline__ double inv_sqrt(double x) {
 }
 
 // All blocks of the (cooperative) launch arrive before any leaves; false in
-// every thread when the wait has not ended after a second.  target counts
+// every thread when the wait has not ended after ctl->wait_ns.  target counts
 // the arrivals since the barrier's reset, modulo 2^32.
 __device__ bool orth_barrier(KCtl* ctl, unsigned target, int* ok) {
   __syncthreads();
   if (threadIdx.x == 0) {
     *ok = 1;
     if (gridDim.x > 1) {
+      const uint64_t limit = ctl->wait_ns;
       __threadfence();
       atomicAdd(&ctl->bar, 1u);
       const uint64_t t0 = now_ns();
@@ -107,7 +107,7 @@ __device__ bool orth_barrier(KCtl* ctl, unsigned target, int* ok) {
       while (true) {
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&ctl->bar) : "memory");
         if ((int)(v - target) >= 0) break;
-        if (now_ns() - t0 > kOrthWaitNs) {
+        if (now_ns() - t0 >= limit) {
           *ok = 0;
           break;
         }
@@ -119,7 +119,10 @@ __device__ bool orth_barrier(KCtl* ctl, unsigned target, int* ok) {
 }
 
 // A wait ran out: the cycle of every segment ends and the solve reports it
-// (one thread).
+// (one thread).  Another block that did pass may be between its read of
+// all_done and its own setting of the loop's condition (end_arnoldi_step), so
+// the condition can end up set: the next pass then finds every segment done
+// and clears it (end_loop).
 __device__ void orth_give_up(SegState* st, KCtl* ctl, int nseg, cudaGraphConditionalHandle cond) {
   for (int s = 0; s < nseg; ++s) {
     st[s].bad = 2;
@@ -127,6 +130,12 @@ __device__ void orth_give_up(SegState* st, KCtl* ctl, int nseg, cudaGraphConditi
   }
   ctl->all_done = 1;
   if (cond) cudaGraphSetConditional(cond, 0);
+}
+
+// Nothing left to do at a launch's start: the loop node (if any) ends here,
+// whatever its condition was left at.
+__device__ __forceinline__ void end_loop(cudaGraphConditionalHandle cond) {
+  if (cond && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(cond, 0);
 }
 
 // Reduce-scatter of NB per-lane values over a warp (NB a power of two):
@@ -267,8 +276,8 @@ __device__ __forceinline__ void mbar_expect(uint64_t* b, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared.b64 _, [%0], %1;" ::"r"(smem_addr(b)), "r"(bytes)
                : "memory");
 }
-// Waits for the phase with the given parity; false after a second.
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, unsigned parity) {
+// Waits for the phase with the given parity; false after `limit` nanoseconds.
+__device__ __forceinline__ bool mbar_wait(uint64_t* b, unsigned parity, uint64_t limit) {
   const uint32_t a = smem_addr(b);
   uint64_t t0 = 0;
   while (true) {
@@ -283,7 +292,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, unsigned parity) {
     if (done) return true;
     const uint64_t t = now_ns();
     if (!t0) t0 = t;
-    if (t - t0 > kOrthWaitNs) return false;
+    if (t - t0 >= limit) return false;
   }
 }
 __device__ __forceinline__ void bulk_copy(void* dst, const void* src, unsigned bytes,
@@ -496,7 +505,7 @@ __global__ void __launch_bounds__(kOneThreads, 1)
   SegState& S = st[0];
   const int j = ctl->j, m = ctl->m, nvec = j + 1;
   const unsigned base = ctl->bar_base;
-  if (mode == ORTH_STEP && S.done) return;
+  if (mode == ORTH_STEP && S.done) return end_loop(cond);
   const int n1 = 2 * nvec + 1, n2 = nvec + 1;  // sums of the first and second reduction
   const int64_t start = (int64_t)blockIdx.x * P.share;
   const int len = (int)(P.n - start < P.share ? P.n - start : P.share);
@@ -599,6 +608,7 @@ constexpr size_t kRingBytes = (size_t)kStages * kGV * kChunk * sizeof(float);
 
 struct Ring {
   uint64_t full[kStages], empty[kStages];
+  uint64_t limit;  // of each wait, ns
 };
 
 // Of kOrthList pieces of the block, those whose segment takes part, in order.
@@ -654,7 +664,7 @@ __device__ __forceinline__ bool ring_fill(const float* Vb, int64_t ld, int64_t s
     const unsigned bytes = 4u * chunk_floats(c0, head, len);
     for (int q = 0; q < nseq; q += kGV) {
       const unsigned s = it % kStages, use = it / kStages;
-      if (use > 0 && !mbar_wait(&R.empty[s], (use - 1) & 1)) return false;
+      if (use > 0 && !mbar_wait(&R.empty[s], (use - 1) & 1, R.limit)) return false;
       const int nv = min(kGV, nseq - q);
       mbar_expect(&R.full[s], bytes * nv);
       for (int k = 0; k < nv; ++k) {
@@ -697,7 +707,7 @@ __device__ __forceinline__ void ring_dot(const float* ring, Ring& R, unsigned& i
     for (int q = 0; q < 8; ++q) {
       if (kGV * q < nseq) {
         const unsigned s = it % kStages;
-        ok = ok && mbar_wait(&R.full[s], (it / kStages) & 1);
+        ok = ok && mbar_wait(&R.full[s], (it / kStages) & 1, R.limit);
         const float* p = ring + (size_t)s * kGV * kChunk;
 #pragma unroll
         for (int k = 0; k < kGV; ++k) {
@@ -748,7 +758,7 @@ __device__ __forceinline__ void ring_upd(const float* ring, Ring& R, unsigned& i
     float acc[4];
     for (int q = 0; q < nseq; q += kGV) {
       const unsigned s = it % kStages;
-      ok = ok && mbar_wait(&R.full[s], (it / kStages) & 1);
+      ok = ok && mbar_wait(&R.full[s], (it / kStages) & 1, R.limit);
       const float* p = ring + (size_t)s * kGV * kChunk;
 #pragma unroll
       for (int k = 0; k < kGV; ++k) {
@@ -794,7 +804,7 @@ __global__ void __launch_bounds__(kManyThreads, 1)
   const bool givens = warp == kOrthWarps + 1;
   const int j = ctl->j, m = ctl->m, nvec = j + 1, nseg = ctl->nseg;
   const unsigned base = ctl->bar_base;
-  if (mode == ORTH_STEP && ctl->all_done) return;
+  if (mode == ORTH_STEP && ctl->all_done) return end_loop(cond);
   const int n1 = 2 * nvec + 1, n2 = nvec + 1;
   double* part1 = P.partial;
   double* part2 = P.partial + (int64_t)P.nslot * 64;
@@ -805,6 +815,7 @@ __global__ void __launch_bounds__(kManyThreads, 1)
       mbar_init(&R.full[s], 1);
       mbar_init(&R.empty[s], kOrthWarps);
     }
+    R.limit = ctl->wait_ns;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   clear_sums(sh, n1);
@@ -1040,7 +1051,7 @@ __global__ void __launch_bounds__(kManyThreads, 1)
     orth_give_up(st, ctl, nseg, cond);
     if (copier)
       for (unsigned k = it > kStages ? it - kStages : 0; k < it; ++k)
-        mbar_wait(&R.full[k % kStages], (k / kStages) & 1);
+        mbar_wait(&R.full[k % kStages], (k / kStages) & 1, kWaitNs);
   }
 }
 
