@@ -890,12 +890,22 @@ __global__ void __launch_bounds__(kManyThreads, 1)
         }
     }
   }
-  if (mode == ORTH_DOT) return;
+  // Before a block ends, its copies have landed.  They have when every wait
+  // for a full stage ended; behind one that ran out, or a copying warp that
+  // gave up, some may be under way, and the shared memory they write to
+  // belongs to the next block.
+  auto land = [&]() {
+    if (f32 && copier && lane == 0)
+      for (unsigned k = it > kStages ? it - kStages : 0; k < it; ++k)
+        mbar_wait(&R.full[k % kStages], (k / kStages) & 1, kWaitNs);
+  };
+  if (mode == ORTH_DOT) return land();
   unsigned bars = 0;
   auto meet = [&]() {
     bars += 1;
     if (orth_barrier(ctl, base + bars * G, &sh.ok)) return true;
     if (tid == 0) orth_give_up(st, ctl, nseg, cond);
+    land();
     return false;
   };
   // the last segment handled ends the step (one thread)
@@ -1006,7 +1016,7 @@ __global__ void __launch_bounds__(kManyThreads, 1)
           }
       }
     }
-    if (mode == ORTH_UPD) return;
+    if (mode == ORTH_UPD) return land();
   }
   // ---- second pass ----------------------------------------------------------
   const int nredo = mode == ORTH_STEP ? *(volatile int*)&ctl->nredo : 1;
@@ -1046,13 +1056,8 @@ __global__ void __launch_bounds__(kManyThreads, 1)
     }
   }
   if (blockIdx.x == 0 && tid == 0 && bars > 0) ctl->bar_base = base + bars * G;
-  // a wait ran out: the solve reports it; the block's copies land first
-  if (!ok && lane == 0) {
-    orth_give_up(st, ctl, nseg, cond);
-    if (copier)
-      for (unsigned k = it > kStages ? it - kStages : 0; k < it; ++k)
-        mbar_wait(&R.full[k % kStages], (k / kStages) & 1, kWaitNs);
-  }
+  if (!ok && lane == 0) orth_give_up(st, ctl, nseg, cond);  // a wait ran out
+  land();
 }
 
 template <typename V>

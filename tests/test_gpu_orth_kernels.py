@@ -42,3 +42,22 @@ def test_a_wait_that_runs_out_is_reported(lib, many, f32):
             assert (out["seg"][:, :2] == [2, 1]).all() and out["ctl"][1] == 1
         else:
             assert (out["seg"][:, :2] == 0).all() and out["ctl"][:2].tolist() == [4, 0]
+
+
+# a limit of 0: the waits for bulk copies run out while the copies are under
+# way; the blocks end behind their copies and a launch after them is clean
+def test_expired_ring_waits_end_behind_their_copies(lib):
+    r = np.random.RandomState(2)
+    lens = [20001, 7, 30002]
+    V = np.concatenate([H.basis(r, 3, k) for k in lens], axis=1)
+    for wait_ns in (0, 10**9):
+        out = H.step(lib, True, H.many(lens, 2048, 8, 3, wait_ns=wait_ns), V)
+        if wait_ns == 0:
+            assert (out["seg"][:, :2] == [2, 1]).all() and out["ctl"][1] == 1
+        else:
+            assert (out["seg"][:, :2] == 0).all() and out["ctl"][:2].tolist() == [4, 0]
+            w, q = out["w"], V[:4]
+            for s, e in zip(np.cumsum([0] + lens[:-1]), np.cumsum(lens)):
+                # FP32 rows of norm 1: entries rounded to 6e-8, a few operations each
+                assert np.abs(q[:, s:e] @ w[s:e]).max() <= 1e-6
+                assert abs(np.linalg.norm(w[s:e]) - 1) <= 1e-6
