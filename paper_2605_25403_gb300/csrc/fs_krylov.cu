@@ -199,23 +199,24 @@ __global__ void __launch_bounds__(kKB) k_seg_update_x(const SegState* st, const 
   constexpr bool pairs = sizeof(V) == 4;
   __shared__ double y[kMaxRestart];
   __shared__ float yh[kMaxRestart], yl[kMaxRestart];
-  __shared__ double H[kMaxRestart * (kMaxRestart + 1)];
+  constexpr int kLd = 33;  // odd: a lane's row starts on a bank of its own
+  __shared__ double H[kMaxRestart * kLd];
   const Tile t = tiles[blockIdx.x];
   const SegState& S = st[t.seg];
   const int k = S.k, m = ctl->m;
   if (k == 0) return;
   for (int i = threadIdx.x >> 5; i < k; i += kKB / 32) {
     const int c = threadIdx.x & 31;
-    if (c < k) H[i * (kMaxRestart + 1) + c] = S.H[i * m + c];
+    if (c < k) H[i * kLd + c] = S.H[i * m + c];
   }
   __syncthreads();
   if (threadIdx.x < 32) {
     const int i = threadIdx.x;
     double g = i < k ? S.g[i] : 0.0;
-    const double r = i < k ? 1.0 / H[i * (kMaxRestart + 1) + i] : 0.0;
+    const double r = i < k ? 1.0 / H[i * kLd + i] : 0.0;
     for (int c = k - 1; c >= 0; --c) {
       const double yc = __shfl_sync(kFull, g * r, c);
-      if (i < c) g -= H[i * (kMaxRestart + 1) + c] * yc;
+      if (i < c) g -= H[i * kLd + c] * yc;
       if (i == c) {
         y[c] = yc;
         yh[c] = (float)yc;

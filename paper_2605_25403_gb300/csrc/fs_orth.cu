@@ -63,7 +63,9 @@ constexpr int kOrthMain = 32 * kOrthWarps;       // threads that work on entries
 constexpr int kOneThreads = kOrthMain + 32;      // k_orth_one: and a Givens warp
 constexpr int kManyThreads = kOrthMain + 64;     // k_orth_many: a copying and a Givens warp
 constexpr double kRedo = 0.01;
-static_assert(kMaxRestart <= 32, "a lane per basis vector");
+// j + 1 <= 31 basis vectors beside w: 2 (j + 1) + 1 sums in slots of 64, and
+// lanes 30 and 31 of the ring's sums hold a_j and w.w
+static_assert(kMaxRestart <= 31, "a lane per basis vector, 64 sums per slot");
 
 template <typename V>
 __device__ __forceinline__ V warp_sum(V v) {

@@ -110,7 +110,7 @@ std::vector<SegState> segments(const Case& c, int done) {
 
 KCtl control(const Case& c, int done) {
   KCtl k{};
-  k.m = 30;
+  k.m = fs::kMaxRestart;
   k.nseg = c.nseg;
   k.j = c.j;
   k.ndone = done ? c.nseg : 0;

@@ -80,3 +80,25 @@ def basis(r, j, n, wnorm=1.0, inside=None):
         inside = 0.5
     w = w / np.linalg.norm(w) * np.sqrt(1 - inside) + q[j + 1] * np.sqrt(inside)
     return np.concatenate([q[:j + 1], wnorm * w[None]])
+
+
+def reference(V, seg0, dtype):
+    """The step on rows of the given type in extended precision: per segment
+    the projection of w onto the others' span, the norm of what is left and
+    that vector normalised; and the Gram correction the earlier steps left
+    (rows and columns below j)."""
+    X = V.astype(dtype).astype(np.longdouble)
+    j = len(V) - 2
+    new, h, E = np.empty_like(X[0]), [], np.zeros((len(seg0) - 1, 32, 32))
+    for s, (a, b) in enumerate(zip(seg0[:-1], seg0[1:])):
+        Q, w = X[:j + 1, a:b], X[j + 1, a:b]
+        G = Q @ Q.T - np.eye(j + 1, dtype=np.longdouble)
+        E[s, :j, :j] = G[:j, :j]
+        c = p = Q @ w
+        for _ in range(12):
+            c = p - G @ c  # (I + G) c = p, G of rounding size
+        r = w - c @ Q
+        nrm = np.sqrt(r @ r)
+        new[a:b] = r / nrm
+        h.append(np.append(c, nrm))
+    return new, np.array(h), E

@@ -61,3 +61,20 @@ def test_expired_ring_waits_end_behind_their_copies(lib):
                 # FP32 rows of norm 1: entries rounded to 6e-8, a few operations each
                 assert np.abs(q[:, s:e] @ w[s:e]).max() <= 1e-6
                 assert abs(np.linalg.norm(w[s:e]) - 1) <= 1e-6
+
+
+# from the first step to the longest basis the kernels hold; FP32 rows carry
+# 6e-8 per entry, and a sum of 31 products of such entries 31 times that
+@pytest.mark.parametrize("f32", [False, True])
+@pytest.mark.parametrize("j", [0, 7, 29, 30])
+@pytest.mark.parametrize("many", [False, True])
+def test_step_against_extended_precision(lib, many, j, f32):
+    r = np.random.RandomState(3)
+    case = H.many([700, 301, 33, 2049], 256, 6, j) if many else H.one(1501, 512, j, LU=1)
+    V = np.concatenate([H.basis(r, j, k) for k in np.diff(case[1])], axis=1)
+    new, h, E = H.reference(V, case[1], np.float32 if f32 else np.float64)
+    out = H.step(lib, f32, case, V, E)
+    u = 6e-8 if f32 else 1.2e-16
+    assert (out["seg"][:, 0] == 0).all() and out["ctl"][0] == j + 1
+    assert np.abs(out["h"] - h).max() <= 20 * u
+    assert np.abs(out["w"] - new).max() <= 100 * u
