@@ -182,18 +182,28 @@ __device__ __forceinline__ void lane_load(const V* p, int e0, int T, int len, bo
 // Dot products of a piece (len entries) with the basis vectors 0 .. nvec - 1
 // (ld apart from base on): part[v] += v . y, with TWO part[nvec + v] += v . z,
 // and after them += y . y.  T threads per group; the groups share the
-// vectors, NB at a time; the warp's sums are taken once per batch.
+// vectors, NB at a time.  FP32 sums run over the 128 products of a warp's
+// chunk and are added in FP64; FP64 ones are taken across the warp once per
+// batch.
 template <typename V, int LE, int NB, bool TWO>
 __device__ __forceinline__ void dot_piece(const V* base, int64_t ld, int nvec, const V* y,
                                           const V* z, int len, int T, double* part) {
+  constexpr bool f32 = sizeof(V) == 4;
+  static_assert(!f32 || LE <= 4, "FP32 sums of at most 128 products");
   const int lane = threadIdx.x & 31, NG = kOrthMain / T;
   const int grp = threadIdx.x / T, t = threadIdx.x - grp * T;
   for (int v0 = grp * NB; v0 < nvec; v0 += NG * NB) {
     const int nb = min(NB, nvec - v0);
     const V* bv = base + (int64_t)v0 * ld;
+    double sd = 0, se = 0, sy = 0;  // the lane's slot: sums of the warp
     V d[NB], e[NB], yy = V(0);
 #pragma unroll
     for (int b = 0; b < NB; ++b) d[b] = e[b] = V(0);
+    auto take = [&]() {
+      sd += (double)warp_transpose_sum<NB, V>(d);
+      if constexpr (TWO) se += (double)warp_transpose_sum<NB, V>(e);
+      if (v0 == 0) sy += (double)warp_sum(yy);
+    };
     for (int c0 = 0; c0 + (t & ~31) < len; c0 += T * LE) {
       const int e0 = c0 + t;
       const bool full = c0 + T * LE <= len;
@@ -203,6 +213,11 @@ __device__ __forceinline__ void dot_piece(const V* base, int64_t ld, int nvec, c
         if (b < nb) lane_load<V, LE>(bv + (int64_t)b * ld, e0, T, len, full, x[b]);
       lane_load<V, LE>(y, e0, T, len, full, w);
       if constexpr (TWO) lane_load<V, LE>(z, e0, T, len, full, u);
+      if constexpr (f32) {
+        yy = V(0);
+#pragma unroll
+        for (int b = 0; b < NB; ++b) d[b] = e[b] = V(0);
+      }
 #pragma unroll
       for (int b = 0; b < NB; ++b)
         if (b < nb) {
@@ -216,22 +231,19 @@ __device__ __forceinline__ void dot_piece(const V* base, int64_t ld, int nvec, c
 #pragma unroll
         for (int k = 0; k < LE; ++k) yy += w[k] * w[k];
       }
+      if constexpr (f32) take();
     }
+    if constexpr (!f32) take();
     constexpr int kShare = 32 / NB;  // lanes holding one slot's sum
     const int slot = lane / kShare;
-    const bool put = lane % kShare == 0 && slot < nb;
-    const V s = warp_transpose_sum<NB, V>(d);
-    if (put) part[v0 + slot] += (double)s;
-    if constexpr (TWO) {
-      const V r = warp_transpose_sum<NB, V>(e);
-      if (put) part[nvec + v0 + slot] += (double)r;
+    if (lane % kShare == 0 && slot < nb) {
+      part[v0 + slot] += sd;
+      if constexpr (TWO) part[nvec + v0 + slot] += se;
     }
-    if (v0 == 0) {
-      yy = warp_sum(yy);
-      if (lane == 0) part[TWO ? 2 * nvec : nvec] += (double)yy;
-    }
+    if (v0 == 0 && lane == 0) part[TWO ? 2 * nvec : nvec] += sy;
   }
 }
+
 // w = (w - sum_v coef[v] v) f over a piece.
 template <typename V, int LU, int NB>
 __device__ __forceinline__ void upd_piece(const V* base, int64_t ld, int nvec, V* w, int len,

@@ -78,3 +78,16 @@ def test_step_against_extended_precision(lib, many, j, f32):
     assert (out["seg"][:, 0] == 0).all() and out["ctl"][0] == j + 1
     assert np.abs(out["h"] - h).max() <= 20 * u
     assert np.abs(out["w"] - new).max() <= 100 * u
+
+
+# FP32 sums run over 128 products and are added in FP64: entries whose sums of
+# up to 128 are exact in FP32 (1 + 2^-22 times powers of two) give an exact
+# projection, where a lane's longer FP32 sum drops the 2^-22
+@pytest.mark.parametrize("T", [512, 256, 64])
+def test_fp32_sums_are_short(lib, T):
+    n = 4096
+    case = H.one(n, 4096, 0, T=T, LU=4)
+    w = np.repeat([1.0, 2.0], n // 2) * (1 + 2.0 ** -22) / 64
+    out = H.step(lib, True, case, np.stack([np.full(n, 1.0 / 64), w]))
+    want = (w / 64).sum()
+    assert abs(out["h"][0, 0] - want) <= 1e-13 * want
