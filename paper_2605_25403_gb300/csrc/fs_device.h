@@ -572,7 +572,8 @@ struct SegState {
   double h2[kMaxRestart + 1];  // coefficients of the running update
   double f;                    // and 1 / ||w|| (orthogonalisation by pieces),
   int act;                     // 0: not active, 1: active, 2: second pass needed
-  float E[32 * 32];  // V^T V - I of the cycle's basis (symmetric)
+  // V^T V - I of the cycle's basis (symmetric), 32 x 32 in the vectors' type
+  double E[32 * 32];
 };
 #ifdef __CUDACC__
 __device__ __forceinline__ bool seg_skipped(const SegSkip& k, int64_t row) {

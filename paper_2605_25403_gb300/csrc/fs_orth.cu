@@ -318,24 +318,33 @@ __device__ __forceinline__ void bulk_copy(void* dst, const void* src, unsigned b
       : "memory");
 }
 
+// A segment's E, held in the type of its vectors.
+template <typename V>
+__host__ __device__ __forceinline__ V* gram(SegState& S) {
+  return reinterpret_cast<V*>(S.E);
+}
+
 // Shared by both kernels.
+template <typename V>
 struct OrthShared {
   double wpart[kOrthWarps][64];  // a warp's sums
   double red[kOrthMain];
   double sum[64];
   double hcol[kMaxRestart + 1];  // the Hessenberg column
-  float E[32 * 33];
-  float c[32];  // E a
-  double f;     // 1 / hn
+  V E[32 * 33];
+  V c[4][32];  // E a (FP64: in four shares of the columns)
+  double f;    // 1 / hn
   int redo, ok;
 };
 
-__device__ __forceinline__ void clear_sums(OrthShared& sh, int ns) {
+template <typename V>
+__device__ __forceinline__ void clear_sums(OrthShared<V>& sh, int ns) {
   for (int i = threadIdx.x; i < kOrthWarps * 64; i += blockDim.x)
     if ((i & 63) < ns) (&sh.wpart[0][0])[i] = 0.0;
 }
 // A slot's first ns sums from the warps' (threads 0 .. ns - 1).
-__device__ __forceinline__ void store_sums(const OrthShared& sh, double* slot, int ns) {
+template <typename V>
+__device__ __forceinline__ void store_sums(const OrthShared<V>& sh, double* slot, int ns) {
   if (threadIdx.x < ns) {
     double s[4] = {0, 0, 0, 0};
 #pragma unroll
@@ -346,7 +355,8 @@ __device__ __forceinline__ void store_sums(const OrthShared& sh, double* slot, i
 
 // sh.sum = the first ns sums added over count slots (64 apart), in a fixed
 // order (whole block).
-__device__ __forceinline__ void reduce_sums(OrthShared& sh, const double* part, int ns,
+template <typename V>
+__device__ __forceinline__ void reduce_sums(OrthShared<V>& sh, const double* part, int ns,
                                             int count) {
   const int tid = threadIdx.x;
   const int parts = kOrthMain / ns, g = tid / ns, s = tid - g * ns;
@@ -383,28 +393,42 @@ __device__ __forceinline__ void reduce_sums(OrthShared& sh, const double* part, 
 // From the sums of the dot pass (sh.sum) and E: c = E a, then h, hn and the
 // decision on a second pass (whole block; sh.hcol, sh.f and sh.redo are
 // valid after the caller's next barrier).  Row j of E goes to S when store.
-__device__ __forceinline__ void first_column(OrthShared& sh, int j, bool force, SegState& S,
+// In FP32 a warp takes a row of E a and adds it over its lanes; in FP64,
+// whose additions over the lanes would cost most of it, a lane takes a row
+// and four warps (one per quarter SM) eight columns each.
+template <typename V>
+__device__ __forceinline__ void first_column(OrthShared<V>& sh, int j, bool force, SegState& S,
                                              bool store) {
+  constexpr bool f32 = sizeof(V) == 4;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nvec = j + 1;
-  const float a = lane < nvec ? (float)sh.sum[lane] : 0.0f;
-  const float e =
-      lane < nvec ? (float)(sh.sum[nvec + lane] - (lane == j ? 1.0 : 0.0)) : 0.0f;
-  if (warp < kOrthWarps) {
+  const V e = lane < nvec ? (V)(sh.sum[nvec + lane] - (lane == j ? 1.0 : 0.0)) : V(0);
+  if (f32 && warp < kOrthWarps) {
+    const V a = lane < nvec ? (V)sh.sum[lane] : V(0);
     for (int i = warp; i < nvec; i += kOrthWarps) {
       // row i of E: E[i][k] for k < j, e_i in column j; row j is e
-      const float ei = __shfl_sync(kFull, e, i);
-      const float r = i == j ? e : lane < j ? sh.E[i * 33 + lane] : lane == j ? ei : 0.0f;
-      const float s = warp_sum(r * a);
-      if (lane == 0) sh.c[i] = s;
+      const V ei = __shfl_sync(kFull, e, i);
+      const V r = i == j ? e : lane < j ? sh.E[i * 33 + lane] : lane == j ? ei : V(0);
+      const V s = warp_sum(r * a);
+      if (lane == 0) sh.c[0][i] = s;
     }
-  } else if (store && lane < nvec) {
-    S.E[lane * 32 + j] = e;
-    S.E[j * 32 + lane] = e;
+  } else if (!f32 && warp < 4) {
+    V s = V(0);
+    for (int k = 8 * warp; k < 8 * warp + 8 && k < nvec; ++k) {
+      const V ek = __shfl_sync(kFull, e, k);
+      const V r = lane == j ? ek : lane > j ? V(0) : k == j ? e : sh.E[lane * 33 + k];
+      s += r * (V)sh.sum[k];
+    }
+    sh.c[warp][lane] = s;
+  } else if (warp >= kOrthWarps && store && lane < nvec) {
+    gram<V>(S)[lane * 32 + j] = e;
+    gram<V>(S)[j * 32 + lane] = e;
   }
   __syncthreads();
   if (warp == 0) {
     const double ad = lane < nvec ? sh.sum[lane] : 0.0;
-    const double h = lane < nvec ? ad - (double)sh.c[lane] : 0.0;
+    double c = (double)sh.c[0][lane];
+    if constexpr (!f32) c = (c + sh.c[1][lane]) + (sh.c[2][lane] + sh.c[3][lane]);
+    const double h = lane < nvec ? ad - c : 0.0;
     const double ww = sh.sum[2 * nvec];
     const double hn2 = ww - warp_sum(ad * h);
     const double f = inv_sqrt(fmax(hn2, 0.0));
@@ -418,7 +442,8 @@ __device__ __forceinline__ void first_column(OrthShared& sh, int j, bool force, 
 }
 
 // After the second pass' sums: h2, and the column with hfirst (warp 0).
-__device__ __forceinline__ void second_column(OrthShared& sh, int nvec, const double* hfirst) {
+template <typename V>
+__device__ __forceinline__ void second_column(OrthShared<V>& sh, int nvec, const double* hfirst) {
   const int lane = threadIdx.x & 31;
   const double h2 = lane < nvec ? sh.sum[lane] : 0.0;
   const double hn2 = sh.sum[nvec] - warp_sum(h2 * h2);
@@ -512,7 +537,7 @@ __global__ void __launch_bounds__(kOneThreads, 1)
   constexpr bool f32 = sizeof(V) == 4;
   constexpr int LE = 4, NB = f32 ? 8 : 2;
   constexpr int NBU = f32 ? (LU == 4 ? 8 : 16) : 8;
-  __shared__ OrthShared sh;
+  __shared__ OrthShared<V> sh;
   __shared__ V coef[32];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool work = warp < kOrthWarps;
@@ -531,9 +556,9 @@ __global__ void __launch_bounds__(kOneThreads, 1)
   clear_sums(sh, n1);
   if (!work && mode < ORTH_DOT)  // E, read while the dot pass runs
     for (int i = 0; i < j; ++i)
-      if (lane < j) sh.E[i * 33 + lane] = S.E[i * 32 + lane];
+      if (lane < j) sh.E[i * 33 + lane] = gram<V>(S)[i * 32 + lane];
   if (mode == ORTH_UPD && !work)
-    for (int i = 0; i < 33; ++i) sh.E[i * 32 + lane] = 0.0f;
+    for (int i = 0; i < 33; ++i) sh.E[i * 32 + lane] = V(0);
   __syncthreads();
   if (mode <= ORTH_DOT) {
     if (work)
@@ -809,7 +834,7 @@ __global__ void __launch_bounds__(kManyThreads, 1)
   constexpr int LE = f32 ? 2 : 4, NB = f32 ? 8 : 2;
   extern __shared__ __align__(128) unsigned char smem[];
   float* ring = reinterpret_cast<float*>(smem);
-  __shared__ OrthShared sh;
+  __shared__ OrthShared<V> sh;
   __shared__ Ring R;
   __shared__ PieceList L;
   __shared__ V coef[32];
@@ -944,7 +969,8 @@ __global__ void __launch_bounds__(kManyThreads, 1)
       }
       if (givens)
         for (int i = 0; i < j; ++i)
-          if (lane < j) sh.E[i * 33 + lane] = mode == ORTH_STEP ? S.E[i * 32 + lane] : 0.0f;
+          if (lane < j) 
+            sh.E[i * 33 + lane] = mode == ORTH_STEP ? gram<V>(S)[i * 32 + lane] : V(0);
       reduce_sums(sh, part1 + (int64_t)P.seg_slot[2 * s] * 64, n1, P.seg_slot[2 * s + 1]);
       first_column(sh, j, mode != ORTH_STEP, S, mode == ORTH_STEP);
       __syncthreads();

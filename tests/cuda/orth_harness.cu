@@ -94,7 +94,7 @@ int plan(const Case& c, const int64_t* seg0, Pool& pool, OrthPlan& o) {
 // The Gram correction of a segment as the kernels of type V hold it.
 template <typename V>
 auto* gram(SegState& S) {
-  return S.E;
+  return fs::gram<V>(S);
 }
 
 std::vector<SegState> segments(const Case& c, int done) {

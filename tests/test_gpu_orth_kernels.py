@@ -91,3 +91,24 @@ def test_fp32_sums_are_short(lib, T):
     out = H.step(lib, True, case, np.stack([np.full(n, 1.0 / 64), w]))
     want = (w / 64).sum()
     assert abs(out["h"][0, 0] - want) <= 1e-13 * want
+
+
+# FP64 vectors: the Gram correction and its product with the sums carry FP64
+# (rows that have lost 1e-6 of their orthogonality; one FP64 rounding each of
+# some 30 products and sums of size 1)
+@pytest.mark.parametrize("many", [False, True])
+def test_fp64_correction_is_fp64(lib, many):
+    r = np.random.RandomState(4)
+    j = 12
+    case = H.many([700, 2049], 256, 6, j) if many else H.one(1501, 512, j)
+    V = np.concatenate([H.basis(r, j, k) for k in np.diff(case[1])], axis=1)
+    for a, b in zip(case[1][:-1], case[1][1:]):
+        V[:j + 1, a:b] += 1e-6 * r.uniform(-1, 1, (j + 1, j + 1)) @ V[:j + 1, a:b]
+    X = V.astype(np.longdouble)
+    _, _, E = H.reference(V, case[1], np.float64)
+    out = H.step(lib, False, case, V, E)
+    for s, (a, b) in enumerate(zip(case[1][:-1], case[1][1:])):
+        Q, p = X[:j + 1, a:b], X[:j + 1, a:b] @ X[j + 1, a:b]
+        G = Q @ Q.T - np.eye(j + 1, dtype=np.longdouble)
+        assert np.abs(out["h"][s, :j + 1] - (p - G @ p)).max() <= 30 * 1.2e-16
+        assert np.abs(out["E"][s, j, :j + 1] - G[j]).max() <= 30 * 1.2e-16
