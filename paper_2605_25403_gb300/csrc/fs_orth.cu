@@ -94,14 +94,13 @@ __device__ __forceinline__ double inv_sqrt(double x) {
 }
 
 // All blocks of the (cooperative) launch arrive before any leaves; false in
-// every thread when the wait has not ended after ctl->wait_ns.  target counts
+// every thread when the wait has not ended after `limit` ns.  target counts
 // the arrivals since the barrier's reset, modulo 2^32.
-__device__ bool orth_barrier(KCtl* ctl, unsigned target, int* ok) {
+__device__ bool orth_barrier(KCtl* ctl, unsigned target, uint64_t limit, int* ok) {
   __syncthreads();
   if (threadIdx.x == 0) {
     *ok = 1;
     if (gridDim.x > 1) {
-      const uint64_t limit = ctl->wait_ns;
       __threadfence();
       atomicAdd(&ctl->bar, 1u);
       const uint64_t t0 = now_ns();
@@ -190,19 +189,26 @@ __device__ __forceinline__ void dot_piece(const V* base, int64_t ld, int nvec, c
                                           const V* z, int len, int T, double* part) {
   constexpr bool f32 = sizeof(V) == 4;
   static_assert(!f32 || LE <= 4, "FP32 sums of at most 128 products");
+  static_assert(32 / NB >= 4, "three lanes of a slot");
   const int lane = threadIdx.x & 31, NG = kOrthMain / T;
   const int grp = threadIdx.x / T, t = threadIdx.x - grp * T;
   for (int v0 = grp * NB; v0 < nvec; v0 += NG * NB) {
     const int nb = min(NB, nvec - v0);
     const V* bv = base + (int64_t)v0 * ld;
-    double sd = 0, se = 0, sy = 0;  // the lane's slot: sums of the warp
     V d[NB], e[NB], yy = V(0);
 #pragma unroll
     for (int b = 0; b < NB; ++b) d[b] = e[b] = V(0);
+    // the warp's sums: of v . y, v . z and y . y in a slot's first three lanes,
+    // so that one FP64 instruction adds all of them
+    constexpr int kShare = 32 / NB;  // lanes holding one slot's sum
+    const int slot = lane / kShare, which = lane % kShare;
+    double acc = 0;
     auto take = [&]() {
-      sd += (double)warp_transpose_sum<NB, V>(d);
-      if constexpr (TWO) se += (double)warp_transpose_sum<NB, V>(e);
-      if (v0 == 0) sy += (double)warp_sum(yy);
+      const V sd = warp_transpose_sum<NB, V>(d);
+      V se = V(0), sy = V(0);
+      if constexpr (TWO) se = warp_transpose_sum<NB, V>(e);
+      if (v0 == 0) sy = warp_sum(yy);
+      acc += (double)(which == 0 ? sd : which == 1 ? se : sy);
     };
     for (int c0 = 0; c0 + (t & ~31) < len; c0 += T * LE) {
       const int e0 = c0 + t;
@@ -234,13 +240,8 @@ __device__ __forceinline__ void dot_piece(const V* base, int64_t ld, int nvec, c
       if constexpr (f32) take();
     }
     if constexpr (!f32) take();
-    constexpr int kShare = 32 / NB;  // lanes holding one slot's sum
-    const int slot = lane / kShare;
-    if (lane % kShare == 0 && slot < nb) {
-      part[v0 + slot] += sd;
-      if constexpr (TWO) part[nvec + v0 + slot] += se;
-    }
-    if (v0 == 0 && lane == 0) part[TWO ? 2 * nvec : nvec] += sy;
+    if (which < (TWO ? 2 : 1) && slot < nb) part[which * nvec + v0 + slot] += acc;
+    if (v0 == 0 && lane == 2) part[TWO ? 2 * nvec : nvec] += acc;
   }
 }
 
@@ -322,6 +323,21 @@ __device__ __forceinline__ void bulk_copy(void* dst, const void* src, unsigned b
 template <typename V>
 __host__ __device__ __forceinline__ V* gram(SegState& S) {
   return reinterpret_cast<V*>(S.E);
+}
+
+// Its rows and columns below j into shared memory (one warp; the loads eight at
+// a time: one by one they outlast the dot pass of a small problem).
+template <typename V>
+__device__ __forceinline__ void load_gram(V* dst, const V* src, int j) {
+  const int lane = threadIdx.x & 31;
+  for (int i = 0; i < j; i += 8) {
+    V v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = i + u < j && lane < j ? src[(i + u) * 32 + lane] : V(0);
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (i + u < j) dst[(i + u) * 33 + lane] = v[u];
+  }
 }
 
 // Shared by both kernels.
@@ -544,6 +560,7 @@ __global__ void __launch_bounds__(kOneThreads, 1)
   SegState& S = st[0];
   const int j = ctl->j, m = ctl->m, nvec = j + 1;
   const unsigned base = ctl->bar_base;
+  const uint64_t limit = ctl->wait_ns;  // of each wait
   if (mode == ORTH_STEP && S.done) return end_loop(cond);
   const int n1 = 2 * nvec + 1, n2 = nvec + 1;  // sums of the first and second reduction
   const int64_t start = (int64_t)blockIdx.x * P.share;
@@ -555,8 +572,7 @@ __global__ void __launch_bounds__(kOneThreads, 1)
   V* vw = bv + (int64_t)nvec * ld;
   clear_sums(sh, n1);
   if (!work && mode < ORTH_DOT)  // E, read while the dot pass runs
-    for (int i = 0; i < j; ++i)
-      if (lane < j) sh.E[i * 33 + lane] = gram<V>(S)[i * 32 + lane];
+    load_gram(sh.E, gram<V>(S), j);
   if (mode == ORTH_UPD && !work)
     for (int i = 0; i < 33; ++i) sh.E[i * 32 + lane] = V(0);
   __syncthreads();
@@ -570,7 +586,7 @@ __global__ void __launch_bounds__(kOneThreads, 1)
   unsigned bars = 0;
   if (mode < ORTH_DOT) {
     bars += 1;
-    if (!orth_barrier(ctl, base + bars * gridDim.x, &sh.ok)) {
+    if (!orth_barrier(ctl, base + bars * gridDim.x, limit, &sh.ok)) {
       if (tid == 0) orth_give_up(st, ctl, 1, cond);
       return;
     }
@@ -606,7 +622,7 @@ __global__ void __launch_bounds__(kOneThreads, 1)
     // second pass: every block took the same decision
     if (redo) {
       bars += 1;
-      if (!orth_barrier(ctl, base + bars * gridDim.x, &sh.ok)) {
+      if (!orth_barrier(ctl, base + bars * gridDim.x, limit, &sh.ok)) {
         if (tid == 0) orth_give_up(st, ctl, 1, cond);
         return;
       }
@@ -843,6 +859,7 @@ __global__ void __launch_bounds__(kManyThreads, 1)
   const bool givens = warp == kOrthWarps + 1;
   const int j = ctl->j, m = ctl->m, nvec = j + 1, nseg = ctl->nseg;
   const unsigned base = ctl->bar_base;
+  const uint64_t limit = ctl->wait_ns;  // of each wait
   if (mode == ORTH_STEP && ctl->all_done) return end_loop(cond);
   const int n1 = 2 * nvec + 1, n2 = nvec + 1;
   double* part1 = P.partial;
@@ -854,7 +871,7 @@ __global__ void __launch_bounds__(kManyThreads, 1)
       mbar_init(&R.full[s], 1);
       mbar_init(&R.empty[s], kOrthWarps);
     }
-    R.limit = ctl->wait_ns;
+    R.limit = limit;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   clear_sums(sh, n1);
@@ -942,7 +959,7 @@ __global__ void __launch_bounds__(kManyThreads, 1)
   unsigned bars = 0;
   auto meet = [&]() {
     bars += 1;
-    if (orth_barrier(ctl, base + bars * G, &sh.ok)) return true;
+    if (orth_barrier(ctl, base + bars * G, limit, &sh.ok)) return true;
     if (tid == 0) orth_give_up(st, ctl, nseg, cond);
     land();
     return false;
@@ -967,10 +984,9 @@ __global__ void __launch_bounds__(kManyThreads, 1)
         if (tid == 0) S.act = 0;
         continue;
       }
-      if (givens)
-        for (int i = 0; i < j; ++i)
-          if (lane < j) 
-            sh.E[i * 33 + lane] = mode == ORTH_STEP ? gram<V>(S)[i * 32 + lane] : V(0);
+      if (givens && mode == ORTH_STEP) load_gram(sh.E, gram<V>(S), j);
+      if (givens && mode != ORTH_STEP)
+        for (int i = 0; i < 33; ++i) sh.E[i * 32 + lane] = V(0);
       reduce_sums(sh, part1 + (int64_t)P.seg_slot[2 * s] * 64, n1, P.seg_slot[2 * s + 1]);
       first_column(sh, j, mode != ORTH_STEP, S, mode == ORTH_STEP);
       __syncthreads();
