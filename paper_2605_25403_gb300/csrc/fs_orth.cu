@@ -476,16 +476,52 @@ __device__ __forceinline__ void second_column(OrthShared<V>& sh, int nvec, const
 // (converged, broken or at the restart length): the segment is then marked
 // done and counted.  One warp: a lane holds a rotation and its operand, so
 // the chain of rotations is one FMA per step.
-__device__ void givens_warp(SegState& S, KCtl* ctl, int j, int m, const double* col) {
-  const int lane = threadIdx.x & 31;
-  const double cs = lane < j ? S.cs[lane] : 1.0, sn = lane < j ? S.sn[lane] : 0.0;
-  const double gj = S.g[j], tol = S.tol_abs;
-  const double b = lane <= j ? col[lane + 1] : 0.0;  // the entry below the diagonal of rotation l
-  const double cb = cs * b;
-  double a = col[0], mine = a;  // the entry rotation l starts from
-  for (int i = 0; i < j; ++i) {
+//
+// The least-squares problem is that of the unit vectors v_l / |v_l|.  The norm
+// by Pythagoras, ww - a.h, has lost the digits that cancel (FP32, hn^2 at 2%
+// of ww: 3e-6 of the norm, where the sums themselves carry 1e-7), but one step
+// later the dot pass finds |v_j|^2 itself, the diagonal of E.  So the rows of
+// the column are scaled by |v_l|, and the entry below the diagonal of the
+// column before, hn |v_j|, and its rotation are brought up to date first.
+// x: the lane's |v_l|^2 - 1.  The rotation's update is a correction of rounding
+// size, relative to what it corrects, so FP32 holds it; its operands are read
+// with the others and its arithmetic runs beside the chain of rotations, which
+// is the launch's critical path on small problems.
+template <typename V>
+__device__ void givens_warp(SegState& S, KCtl* ctl, int j, int m, const double* col, V x) {
+  const int lane = threadIdx.x & 31, p = j > 0 ? j - 1 : 0;
+  double cs = lane < j ? S.cs[lane] : 1.0, sn = lane < j ? S.sn[lane] : 0.0;
+  double gj = S.g[j], gp = S.g[p], hp = S.H[p * m + p];
+  const double tol = S.tol_abs;
+  const V off = lane <= j ? x * (V(0.5) - V(0.125) * x) : V(0);  // |v_l| - 1
+  const double h = lane <= j + 1 ? col[lane] : 0.0, hl = h + h * (double)off;
+  // b -> b (1 + d) in the rotation before: den^2 = a^2 + b^2 grows by 1 + 2 q
+  const float d = (float)__shfl_sync(kFull, off, j), s0 = __shfl_sync(kFull, (float)sn, p);
+  const float q = s0 * s0 * (d + 0.5f * d * d), r = q * (1.5f * q - 1.0f);  // 1/sqrt(1+2q) - 1
+  const double dc = (double)r, ds = (double)(d + r + d * r);
+  // the entry below the diagonal of rotation l, and the one it starts from
+  const double b = __shfl_down_sync(kFull, hl, 1);
+  double cb = cs * b;
+  double a = __shfl_sync(kFull, hl, 0), mine = a;
+  for (int i = 0; i < j - 1; ++i) {
     a = fma(-__shfl_sync(kFull, sn, i), a, __shfl_sync(kFull, cb, i));
     if (lane == i + 1) mine = a;
+  }
+  if (j > 0) {
+    if (lane == p) {
+      cs += cs * dc;
+      sn += sn * ds;
+      cb = cs * b;
+      S.cs[p] = cs;
+      S.sn[p] = sn;
+    }
+    gj += gj * ds;
+    a = fma(-__shfl_sync(kFull, sn, p), a, __shfl_sync(kFull, cb, p));
+    if (lane == j) mine = a;
+    if (lane == 0) {
+      S.g[p] = gp + gp * dc;
+      S.H[p * m + p] = hp + hp * (double)(q - 0.5f * q * q);
+    }
   }
   const double bl = __shfl_sync(kFull, b, j);
   // the new rotation: c = a / den, s = b / den, den = sqrt(a^2 + b^2), the
@@ -592,16 +628,19 @@ __global__ void __launch_bounds__(kOneThreads, 1)
     }
   }
   bool redo = true;
+  V vsq = V(0);  // |v_lane|^2 - 1
   if (mode != ORTH_FIN) {
     reduce_sums(sh, part1, n1, gridDim.x);
     clear_sums(sh, n2);
     first_column(sh, j, mode != ORTH_STEP, S, owner && mode == ORTH_STEP);
     __syncthreads();
     redo = sh.redo != 0;
+    if (!work && lane <= j) 
+      vsq = lane < j ? sh.E[lane * 34] : (V)(sh.sum[nvec + j] - 1.0);
     if (work && lane < nvec) coef[lane] = (V)sh.hcol[lane];  // every warp the same values
     if (!work && owner && mode == ORTH_STEP) {
       if (!redo) {
-        givens_warp(S, ctl, j, m, sh.hcol);
+        givens_warp(S, ctl, j, m, sh.hcol, vsq);
         if (lane == 0) end_arnoldi_step(ctl, j, m, cond);
       } else if (lane < nvec) {
         S.h2[lane] = sh.hcol[lane];  // the first pass' share of the column
@@ -635,7 +674,7 @@ __global__ void __launch_bounds__(kOneThreads, 1)
   __syncthreads();
   if (work && lane < nvec) coef[lane] = (V)sh.sum[lane];
   if (!work && owner && mode == ORTH_STEP) {
-    givens_warp(S, ctl, j, m, sh.hcol);
+    givens_warp(S, ctl, j, m, sh.hcol, vsq);
     if (lane == 0) end_arnoldi_step(ctl, j, m, cond);
   }
   if (work) {
@@ -1009,8 +1048,9 @@ __global__ void __launch_bounds__(kManyThreads, 1)
         if (act == 2) continue;
         if (act == 1) {
           if (lane <= nvec) sh.hcol[lane] = S.h2[lane];
+          const V vsq = lane <= j ? gram<V>(S)[lane * 33] : V(0);
           __syncwarp();
-          givens_warp(S, ctl, j, m, sh.hcol);
+          givens_warp(S, ctl, j, m, sh.hcol, vsq);
         }
         if (lane == 0) count_segment();
         __syncwarp();
@@ -1090,7 +1130,8 @@ __global__ void __launch_bounds__(kManyThreads, 1)
         if (lane == 0) S.f = sh.f;
       }
       if (givens && mode == ORTH_STEP) {
-        givens_warp(S, ctl, j, m, sh.hcol);
+        const V vsq = lane <= j ? gram<V>(S)[lane * 33] : V(0);
+        givens_warp(S, ctl, j, m, sh.hcol, vsq);
         if (lane == 0) count_segment();
       }
     }

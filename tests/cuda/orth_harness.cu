@@ -125,9 +125,11 @@ KCtl control(const Case& c, int done) {
 // One Arnoldi step's orthogonalisation of V[j + 1] against V[0..j] (rows of
 // length n).  E: per segment the 32 x 32 Gram correction, in and out.
 // h: per segment 33 entries, its Hessenberg column before the new rotation.
+// state: the segments' records, used as they are when resume; rot: per
+// segment the cosine and sine of the rotation before this step's.
 template <typename V>
 int step(const Case& c, const int64_t* seg0, const double* Vin, double* E, double* w, double* h,
-         int32_t* seg_out, int32_t* ctl_out) {
+         int32_t* seg_out, int32_t* ctl_out, void* state, int resume, double* rot) {
   Pool pool;
   OrthPlan o;
   if (int rc = plan<V>(c, seg0, pool, o)) return rc;
@@ -138,8 +140,9 @@ int step(const Case& c, const int64_t* seg0, const double* Vin, double* E, doubl
     for (int64_t i = 0; i < c.n; ++i) hv[r * ld + i] = (V)Vin[r * c.n + i];
   V* dV = pool.up(hv);
   std::vector<SegState> st = segments(c, 0);
+  if (resume) memcpy((void*)st.data(), state, sizeof(SegState) * c.nseg);
   for (int s = 0; s < c.nseg; ++s)
-    for (int i = 0; i < 1024; ++i) gram<V>(st[s])[i] = E[1024 * s + i];
+    for (int i = 0; i < 1024 && !resume; ++i) gram<V>(st[s])[i] = E[1024 * s + i];
   SegState* dst = pool.up(st);
   KCtl k = control(c, 0);
   KCtl* dk = pool.up(std::vector<KCtl>{k});
@@ -148,6 +151,7 @@ int step(const Case& c, const int64_t* seg0, const double* Vin, double* E, doubl
   cudaMemcpy(hv.data(), dV, sizeof(V) * hv.size(), cudaMemcpyDeviceToHost);
   cudaMemcpy(st.data(), dst, sizeof(SegState) * c.nseg, cudaMemcpyDeviceToHost);
   cudaMemcpy(&k, dk, sizeof(k), cudaMemcpyDeviceToHost);
+  memcpy(state, st.data(), sizeof(SegState) * c.nseg);
   for (int64_t i = 0; i < c.n; ++i) w[i] = (double)hv[(rows - 1) * ld + i];
   for (int s = 0; s < c.nseg; ++s) {
     const SegState& S = st[s];
@@ -156,6 +160,8 @@ int step(const Case& c, const int64_t* seg0, const double* Vin, double* E, doubl
     const double den = S.H[c.j * k.m + c.j];
     h[33 * s + c.j] = S.cs[c.j] * den;
     h[33 * s + c.j + 1] = S.sn[c.j] * den;
+    rot[2 * s] = c.j > 0 ? S.cs[c.j - 1] : 1.0;
+    rot[2 * s + 1] = c.j > 0 ? S.sn[c.j - 1] : 0.0;
     const int32_t out[4] = {S.bad, S.done, S.act, S.k};
     std::copy(out, out + 4, seg_out + 4 * s);
   }
@@ -217,12 +223,15 @@ int loop(const Case& c, const int64_t* seg0, int max_pass, int* passes) {
 }  // namespace
 
 extern "C" {
+int orth_state_size() { return (int)sizeof(SegState); }
 int orth_step(int f32, const void* c, const int64_t* seg0, const double* V, double* E, double* w,
-              double* h, int32_t* seg_out, int32_t* ctl_out) {
-  return f32 ? step<float>(*(const Case*)c, seg0, V, E, w, h, seg_out, ctl_out)
-             : step<double>(*(const Case*)c, seg0, V, E, w, h, seg_out, ctl_out);
+              double* h, int32_t* seg_out, int32_t* ctl_out, void* state, int resume,
+              double* rot) {
+  return f32 ? step<float>(*(const Case*)c, seg0, V, E, w, h, seg_out, ctl_out, state, resume, rot)
+             : step<double>(*(const Case*)c, seg0, V, E, w, h, seg_out, ctl_out, state, resume, rot);
 }
 int orth_loop(int f32, const void* c, const int64_t* seg0, int max_pass, int* passes) {
-  return f32 ? loop<float>(*(const Case*)c, seg0, max_pass, passes) : loop<double>(*(const Case*)c, seg0, max_pass, passes);
+  return f32 ? loop<float>(*(const Case*)c, seg0, max_pass, passes)
+             : loop<double>(*(const Case*)c, seg0, max_pass, passes);
 }
 }

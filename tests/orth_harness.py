@@ -47,20 +47,24 @@ def many(lens, piece, blocks, j, T=512, wait_ns=10**9, absent=0):
                 n=int(seg0[-1]), share=0, wait_ns=wait_ns), seg0
 
 
-def step(lib, f32, case, V, E=None):
+def step(lib, f32, case, V, E=None, state=None):
     """One step on the rows V (j + 2 of them): the new vector, per segment the
-    Hessenberg column, the Gram correction and (bad, done, act, k); and
-    (j, all_done, nredo, arrivals)."""
+    Hessenberg column, the Gram correction, (bad, done, act, k), the rotation
+    before this step's and the segments' records (a later step's `state`, which
+    then holds E); and (j, all_done, nredo, arrivals)."""
     c, seg0 = case
     V = np.ascontiguousarray(V, dtype=np.float64)
     assert V.shape == (c.j + 2, c.n)
     E = np.zeros((c.nseg, 32, 32)) if E is None else np.array(E, dtype=np.float64)
     w, h = np.empty(c.n), np.zeros((c.nseg, 33))
     seg, ctl = np.zeros((c.nseg, 4), dtype=np.int32), np.zeros(4, dtype=np.int32)
+    resume = state is not None
+    state = state.copy() if resume else np.zeros(c.nseg * lib.orth_state_size(), dtype=np.uint8)
+    rot = np.zeros((c.nseg, 2))
     rc = lib.orth_step(int(f32), ctypes.byref(c), _ptr(seg0), _ptr(V), _ptr(E), _ptr(w), _ptr(h),
-                       _ptr(seg), _ptr(ctl))
+                       _ptr(seg), _ptr(ctl), _ptr(state), int(resume), _ptr(rot))
     assert rc == 0, rc
-    return dict(w=w, h=h[:, :c.j + 2], E=E, seg=seg, ctl=ctl)
+    return dict(w=w, h=h[:, :c.j + 2], E=E, seg=seg, ctl=ctl, rot=rot, state=state)
 
 
 def loop_passes(lib, f32, case, max_pass):

@@ -93,7 +93,8 @@ def test_fp32_sums_are_short(lib, T):
     assert abs(out["h"][0, 0] - want) <= 1e-13 * want
 
 
-# FP64 vectors: the Gram correction and its product with the sums carry FP64
+# FP64 vectors: the Gram correction and its product with the sums carry FP64;
+# the column is that of the unit vectors
 # (rows that have lost 1e-6 of their orthogonality; one FP64 rounding each of
 # some 30 products and sums of size 1)
 @pytest.mark.parametrize("many", [False, True])
@@ -110,5 +111,34 @@ def test_fp64_correction_is_fp64(lib, many):
     for s, (a, b) in enumerate(zip(case[1][:-1], case[1][1:])):
         Q, p = X[:j + 1, a:b], X[:j + 1, a:b] @ X[j + 1, a:b]
         G = Q @ Q.T - np.eye(j + 1, dtype=np.longdouble)
-        assert np.abs(out["h"][s, :j + 1] - (p - G @ p)).max() <= 30 * 1.2e-16
+        nu = np.sqrt(1 + np.diag(G))
+        assert np.abs(out["h"][s, :j + 1] - nu * (p - G @ p)).max() <= 30 * 1.2e-16
         assert np.abs(out["E"][s, j, :j + 1] - G[j]).max() <= 30 * 1.2e-16
+
+
+# The norm by Pythagoras loses the digits that cancel; a step later the dot
+# pass finds the norm itself and the rotation is brought up to date: tangent
+# hn |v_{j+1}| / (h_j |v_j|), to the 2 x 128 products' rounding of the sums
+# (FP32: 9 operations of 6e-8 on partial sums, averaged over n / 128 of them)
+@pytest.mark.parametrize("f32", [False, True])
+@pytest.mark.parametrize("many", [False, True])
+def test_rotation_takes_the_norm_of_the_stored_vector(lib, many, f32):
+    j, n = 11, 2000
+    worst = 0.0
+    for seed in range(6):
+        r = np.random.RandomState(seed)
+        first = H.many([n], 256, 6, j) if many else H.one(n, 512, j)
+        V = H.basis(r, j, n, inside=0.012)
+        _, _, E = H.reference(V, first[1], np.float32 if f32 else np.float64)
+        out = H.step(lib, f32, first, V, E)
+        assert out["seg"][0, 2] != 2  # no second pass
+        c, s = out["h"][0, j], out["h"][0, j + 1]
+        x = out["w"].astype(np.longdouble)
+        norm = np.sqrt(x @ x)
+        worst = max(worst, abs(float(norm) - 1))
+        then = H.many([n], 256, 6, j + 1) if many else H.one(n, 512, j + 1)
+        W = np.concatenate([V[:j + 1], out["w"][None], r.standard_normal((1, n)) / np.sqrt(n)])
+        rot = H.step(lib, f32, then, W, state=out["state"])["rot"][0]
+        want = s / c * float(norm)
+        assert abs(rot[1] / rot[0] / want - 1) <= (9 * 6e-8 / np.sqrt(n / 128) if f32 else 3e-15)
+    assert worst > (1e-7 if f32 else 1e-15)  # the norms were off
