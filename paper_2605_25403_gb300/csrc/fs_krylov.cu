@@ -164,41 +164,35 @@ __global__ void __launch_bounds__(kKB) k_seg_scale(JVec<V> xv, const Tile* tiles
   for (int e = threadIdx.x; e < t.len; e += kKB) x[t.start + e] *= f;
 }
 
-// A sum kept as an unevaluated pair of FP32 numbers (48 bits): s += z y with
-// y = yh + yl given as such a pair (Dekker's two-sum, Numer. Math. 18, 1971;
-// the product's rounding error by an FMA).
-struct Pair {
-  float hi = 0.0f, lo = 0.0f;
-  __device__ __forceinline__ void add(float z, float yh, float yl) {
-    // (the _rn forms keep the compiler from contracting them into FMAs)
-    const float p = __fmul_rn(z, yh), e = fmaf(z, yh, -p);
-    const float t = __fadd_rn(hi, p), b = __fsub_rn(t, hi);
-    const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, b)), __fsub_rn(p, b));
-    lo += err + fmaf(z, yl, e);
-    hi = t;
-  }
-};
+// z 2^-896 in FP64, from the bits of a finite z: an exponent field 896 lower is
+// the same field, so the mantissa only moves (zeros and FP32 denormals
+// included; both scales cancel exactly in a product with y 2^896).  Three
+// integer operations where the conversion instruction takes as long as an
+// FP64 FMA, 64 cycles of a quarter SM per warp.
+__device__ __forceinline__ double widen(float z) {
+  const unsigned b = __float_as_uint(z);
+  return __hiloint2double((int)((b & 0x80000000u) | ((b & 0x7fffffffu) >> 3)), (int)(b << 29));
+}
+__device__ __forceinline__ bool finite_bits(float z) {
+  return (__float_as_uint(z) & 0x7f800000u) != 0x7f800000u;
+}
 
 // y = H(0:k,0:k)^-1 g(0:k) of the tile's segment, then x += Z y.
 //
 // The back substitution runs in one warp, a lane per unknown with the
 // reciprocals of the diagonal taken beforehand, from the triangle in shared
 // memory (one thread walking it through global memory took most of the
-// kernel's time on small vectors).  The sums over the directions run in FP64
-// for FP64 vectors.  For FP32 ones, whose result is rounded to FP32, they
-// run in pairs of FP32 numbers: ten FP32 operations per product where an
-// FP64 FMA and a conversion cost 128 cycles of a quarter SM.  Per cycle on
-// GB300, 24 directions or so: 78 -> 35 us on the 512x96 channel, 418 -> 163 us
-// on the 48^3 cube (286 MB of directions: 44 us at 6.6 TB/s), 209 -> 81 us on
-// the batch of 96 squares, 48 -> 25 us on the FP64 8^2 square.
+// kernel's time on small vectors).  The sums over the directions run in FP64,
+// FP32 directions widened by their bits (unless one is not finite, or a
+// coefficient is 2^127 or more): FP64 arithmetic is what bounds the kernel.
 template <typename V, typename X>
 __global__ void __launch_bounds__(kKB) k_seg_update_x(const SegState* st, const KCtl* ctl,
                                                       const V* __restrict__ Z, int64_t n,
                                                       const Tile* tiles, X* __restrict__ x) {
   pdl_wait();
-  constexpr bool pairs = sizeof(V) == 4;
-  __shared__ double y[kMaxRestart];
-  __shared__ float yh[kMaxRestart], yl[kMaxRestart];
+  constexpr bool f32 = sizeof(V) == 4;
+  __shared__ double y[kMaxRestart], ys[kMaxRestart];  // y, y 2^896
+  __shared__ int by_bits;
   constexpr int kLd = 33;  // odd: a lane's row starts on a bank of its own
   __shared__ double H[kMaxRestart * kLd];
   const Tile t = tiles[blockIdx.x];
@@ -212,49 +206,44 @@ __global__ void __launch_bounds__(kKB) k_seg_update_x(const SegState* st, const 
   __syncthreads();
   if (threadIdx.x < 32) {
     const int i = threadIdx.x;
-    double g = i < k ? S.g[i] : 0.0;
+    double g = i < k ? S.g[i] : 0.0, mine = 0.0;
     const double r = i < k ? 1.0 / H[i * kLd + i] : 0.0;
     for (int c = k - 1; c >= 0; --c) {
       const double yc = __shfl_sync(kFull, g * r, c);
       if (i < c) g -= H[i * kLd + c] * yc;
-      if (i == c) {
-        y[c] = yc;
-        yh[c] = (float)yc;
-        yl[c] = (float)(yc - (double)yh[c]);
-      }
+      if (i == c) mine = yc;
     }
+    if (i < k) {
+      y[i] = mine;
+      ys[i] = scalbn(mine, 896);
+    }
+    const bool fit = __all_sync(kFull, fabs(mine) < 0x1p127);
+    if (i == 0) by_bits = fit;
   }
   __syncthreads();
+  const bool bits = f32 && by_bits;
   for (int e = threadIdx.x; e < t.len; e += kKB) {
     const int64_t i = t.start + e;
     // four directions at a time into separate sums (independent loads)
+    double s[4] = {0, 0, 0, 0};
     int c = 0;
-    if constexpr (pairs) {
-      Pair s[4];
-      for (; c + 4 <= k; c += 4) {
-        float z[4];
+    for (; c + 4 <= k; c += 4) {
+      V z[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) z[u] = (float)Z[(int64_t)(c + u) * n + i];
+      for (int u = 0; u < 4; ++u) z[u] = Z[(int64_t)(c + u) * n + i];
+      if constexpr (f32) {
+        if (bits && finite_bits(z[0]) && finite_bits(z[1]) && finite_bits(z[2]) &&
+            finite_bits(z[3])) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) s[u].add(z[u], yh[c + u], yl[c + u]);
+          for (int u = 0; u < 4; ++u) s[u] += ys[c + u] * widen(z[u]);
+          continue;
+        }
       }
-      for (; c < k; ++c) s[0].add((float)Z[(int64_t)c * n + i], yh[c], yl[c]);
 #pragma unroll
-      for (int u = 1; u < 4; ++u) {
-        s[0].add(s[u].hi, 1.0f, 0.0f);
-        s[0].lo += s[u].lo;
-      }
-      s[0].add((float)x[i], 1.0f, 0.0f);
-      x[i] = (X)(s[0].hi + s[0].lo);
-    } else {
-      double s[4] = {0, 0, 0, 0};
-      for (; c + 4 <= k; c += 4) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) s[u] += y[c + u] * (double)Z[(int64_t)(c + u) * n + i];
-      }
-      for (; c < k; ++c) s[0] += y[c] * (double)Z[(int64_t)c * n + i];
-      x[i] = (X)((double)x[i] + ((s[0] + s[1]) + (s[2] + s[3])));
+      for (int u = 0; u < 4; ++u) s[u] += y[c + u] * (double)z[u];
     }
+    for (; c < k; ++c) s[0] += y[c] * (double)Z[(int64_t)c * n + i];
+    x[i] = (X)((double)x[i] + ((s[0] + s[1]) + (s[2] + s[3])));
   }
 }
 
