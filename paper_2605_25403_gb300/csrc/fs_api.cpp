@@ -449,18 +449,18 @@ SellLayout sell_layout(const HostCsr& H, double uniform_slack = 0.0,
 
 // Values of a CSR matrix with dimv values per entry (vals, entry-major) in
 // the SELL-32 layout L: component c of slot u of row 32 s + t at
-// (off[s] + 32 u) dimv + 32 c + t; padding slots hold 0.  A row's entries and
-// its slots are both in column order.
+// (off[s] + 32 u) dimv + 32 c + t; padding slots hold -0.0, zero entries 0.0.
+// A row's entries and its slots are both in column order.
 template <typename T>
 std::vector<T> sell_values(const HostCsr& H, const SellLayout& L, const double* vals, int dimv) {
-  std::vector<T> v(L.off.back() * dimv, T(0));
+  std::vector<T> v(L.off.back() * dimv, T(-0.0));
   for (int64_t r = 0; r < H.nrow; ++r) {
     const int64_t sl = r >> 5, t = r & 31, w = (L.off[sl + 1] - L.off[sl]) / 32;
     int64_t k = H.rowptr[r];
     for (int64_t u = 0; u < w && k < H.rowptr[r + 1]; ++u) {
       if (L.ci[L.off[sl] + 32 * u + t] != H.col[k]) continue;
       for (int c = 0; c < dimv; ++c)
-        v[(L.off[sl] + 32 * u) * dimv + 32 * c + t] = (T)vals[k * dimv + c];
+        v[(L.off[sl] + 32 * u) * dimv + 32 * c + t] = (T)vals[k * dimv + c] + T(0.0);
       ++k;
     }
   }

@@ -67,8 +67,10 @@ struct DCsr {
 
 // Sliced ELLPACK with slices of 32 rows (one thread per row): the entries of
 // row 32 s + t sit at off[s] + 32 u + t for the slot u < (off[s+1] - off[s]) / 32,
-// so a warp's loads of one slot are contiguous.  Slots past a row's length
-// hold coefficient 0 and a valid column.
+// so a warp's loads of one slot are contiguous.  Slots a row does not use hold
+// the coefficient -0.0 and a valid column; the row's own entries are never
+// -0.0, so that a product can leave the others out where 0 x Inf would matter
+// (a run's padding columns belong to other rows' stencils).
 //
 // Columns.  Consecutive rows of a structured mesh have the same stencil
 // shifted by one, so a slice's slots can be laid out by column offset: in a
@@ -282,7 +284,7 @@ void launch_spmv_full(const DOp<T>& op, JVec<const V> x, const V* b, JVec<V> y,
 
 // Scalar CSR values (row pointers rp, columns ci) into the SELL-32 layout L
 // (its offsets and columns): out64 (and out32 when not null) receive the
-// matrix, zeros in the slots a row does not use.
+// matrix, -0.0 in the slots a row does not use.
 void launch_csr_to_sell(const DSell<double>& L, const int32_t* rp, const int32_t* ci,
                         const double* in, double* out64, float* out32, cudaStream_t s);
 

@@ -41,6 +41,15 @@ __device__ __forceinline__ V group_sum(V v) {
   return v;
 }
 
+// A padding slot of a SELL-32 operator (DSell).  The FP64 saddle-point product,
+// which fs_apply_operator exposes, leaves them out: an entry of x that is not
+// finite reaches the rows that couple to it and no others.  Elsewhere the
+// vectors' norms are taken, which such an entry makes non-finite anyway.
+__device__ __forceinline__ bool is_padding(double a) {
+  return __double_as_longlong(a) == (long long)0x8000000000000000ull;
+}
+__device__ __forceinline__ constexpr bool is_padding(float) { return false; }
+
 // Row loops take kU slots at a time (loads issued before the FMAs); padding
 // slots have coefficient 0 and a valid column.  The FP32 saddle-point SpMV
 // takes kUSpmv (deeper groups measured faster there, cube 48^3: 0.115 ->
@@ -142,6 +151,7 @@ __device__ __forceinline__ void spmv_velocity(const DOp<T>& op, const V* __restr
 #pragma unroll
         for (int u = 0; u < kUS; ++u) {
           if (skip_padding<V>() && k + u >= hi) break;
+          if (is_padding(a[u])) continue;
 #pragma unroll
           for (int c = 0; c < DIM; ++c) acc[c] += a[u] * g[u][c];
         }
@@ -168,6 +178,7 @@ __device__ __forceinline__ void spmv_velocity(const DOp<T>& op, const V* __restr
 #pragma unroll
       for (int u = 0; u < kU; ++u) {
         if (skip_padding<V>() && k + u >= hi) break;
+        if (is_padding(bv[u][0])) continue;
 #pragma unroll
         for (int c = 0; c < DIM; ++c) acc[c] -= bv[u][c] * p[u];
       }
@@ -202,6 +213,7 @@ __device__ __forceinline__ V spmv_pressure(const DOp<T>& op, const V* __restrict
 #pragma unroll
       for (int u = 0; u < kUS; ++u) {
         if (skip_padding<V>() && k + u >= hi) break;
+        if (is_padding(bv[u][0])) continue;
 #pragma unroll
         for (int c = 0; c < DIM; ++c) acc += bv[u][c] * g[u][c];
       }
@@ -293,7 +305,7 @@ __global__ void __launch_bounds__(32 * W) k_spmv_split(DOp<T> op, JVec<const V> 
 
 // CSR -> SELL-32 value scatter, one thread per row: the row's entries and its
 // slots are both in column order, so one walk over the slots places them
-// (padding slots, whose column is not the next entry's, get 0).
+// (padding slots, whose column is not the next entry's, get -0.0).
 __global__ void k_csr_to_sell(DSell<double> L, const int32_t* __restrict__ rp,
                               const int32_t* __restrict__ ci, const double* __restrict__ in,
                               double* __restrict__ out64, float* __restrict__ out32) {
@@ -305,8 +317,8 @@ __global__ void k_csr_to_sell(DSell<double> L, const int32_t* __restrict__ rp,
   R.with_columns(L, [&](auto col, int shift) {
     int32_t k = rp[r];
     for (int u = 0; u < R.w; ++u) {
-      double v = 0.0;
-      if (k < e && ci[k] == col(u) + shift) v = in[k++];
+      double v = -0.0;
+      if (k < e && ci[k] == col(u) + shift) v = in[k++] + 0.0;
       out64[base + 32 * u] = v;
       if (out32) out32[base + 32 * u] = (float)v;
     }
