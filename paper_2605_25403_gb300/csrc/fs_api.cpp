@@ -2704,7 +2704,7 @@ int fs_apply_operator(fs_problem* P, const double* x, double* y) {
   FS_TRY(nat_buffers(P));
   launch_dofs_perm(P->dm, P->nat, x, P->natbuf, 0, P->stream);
   launch_spmv_full<double, double>(P->p64.op, P->natbuf, nullptr, P->natbuf2, 0, nullptr,
-                                   P->stream);
+                                   P->stream, false, /*exact=*/true);
   launch_dofs_perm(P->dm, P->nat, P->natbuf2, y, 1, P->stream);
   return check_launch("fs_apply_operator");
 }

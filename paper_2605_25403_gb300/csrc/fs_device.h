@@ -276,11 +276,13 @@ struct DOp {
 };
 
 // y = K x (resid == 0) or y = b - K x (resid == 1); vectors of type V.
+// exact (FP64): the padding slots take no part, not even as 0 x Inf.
 // seg: skip the rows of converged segments (the Arnoldi step's product;
 // residuals and timing runs take every row).
 template <typename T, typename V>
 void launch_spmv_full(const DOp<T>& op, JVec<const V> x, const V* b, JVec<V> y,
-                      int resid, const int* skip, cudaStream_t s, bool seg = false);
+                      int resid, const int* skip, cudaStream_t s, bool seg = false,
+                      bool exact = false);
 
 // Scalar CSR values (row pointers rp, columns ci) into the SELL-32 layout L
 // (its offsets and columns): out64 (and out32 when not null) receive the

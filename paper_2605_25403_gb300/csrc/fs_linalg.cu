@@ -41,14 +41,18 @@ __device__ __forceinline__ V group_sum(V v) {
   return v;
 }
 
-// A padding slot of a SELL-32 operator (DSell).  The FP64 saddle-point product,
-// which fs_apply_operator exposes, leaves them out: an entry of x that is not
-// finite reaches the rows that couple to it and no others.  Elsewhere the
-// vectors' norms are taken, which such an entry makes non-finite anyway.
-__device__ __forceinline__ bool is_padding(double a) {
-  return __double_as_longlong(a) == (long long)0x8000000000000000ull;
+// A padding slot of a SELL-32 operator (DSell).  fs_apply_operator's product
+// (EXACT) leaves them out: an entry of x that is not finite reaches the rows
+// that couple to it and no others.  The solver's products take them as zeros,
+// because it takes its vectors' norms, which such an entry makes non-finite
+// anyway, and the test of every slot costs 2 to 6% (33^3 cube 74.8 -> 77.2 us,
+// 300x60 channel 9.5 -> 10.2).
+template <bool EXACT, typename V>
+__device__ __forceinline__ bool left_out(V a) {
+  if constexpr (EXACT && sizeof(V) == 8)
+    return __double_as_longlong(a) == (long long)0x8000000000000000ull;
+  return false;
 }
-__device__ __forceinline__ constexpr bool is_padding(float) { return false; }
 
 // Row loops take kU slots at a time (loads issued before the FMAs); padding
 // slots have coefficient 0 and a valid column.  The FP32 saddle-point SpMV
@@ -126,7 +130,7 @@ __device__ __forceinline__ void slot_share(int w, int part, int parts, int& lo, 
 }
 
 // acc += (A u - BT p) over one share of a velocity row's slots.
-template <typename T, typename V, int DIM, int kUS>
+template <typename T, typename V, int DIM, int kUS, bool EXACT>
 __device__ __forceinline__ void spmv_velocity(const DOp<T>& op, const V* __restrict__ x,
                                               int64_t row, int part, int parts, V (&acc)[DIM]) {
   const int64_t n2 = op.n2;
@@ -151,7 +155,7 @@ __device__ __forceinline__ void spmv_velocity(const DOp<T>& op, const V* __restr
 #pragma unroll
         for (int u = 0; u < kUS; ++u) {
           if (skip_padding<V>() && k + u >= hi) break;
-          if (is_padding(a[u])) continue;
+          if (left_out<EXACT>(a[u])) continue;
 #pragma unroll
           for (int c = 0; c < DIM; ++c) acc[c] += a[u] * g[u][c];
         }
@@ -178,7 +182,7 @@ __device__ __forceinline__ void spmv_velocity(const DOp<T>& op, const V* __restr
 #pragma unroll
       for (int u = 0; u < kU; ++u) {
         if (skip_padding<V>() && k + u >= hi) break;
-        if (is_padding(bv[u][0])) continue;
+        if (left_out<EXACT>(bv[u][0])) continue;
 #pragma unroll
         for (int c = 0; c < DIM; ++c) acc[c] -= bv[u][c] * p[u];
       }
@@ -187,7 +191,7 @@ __device__ __forceinline__ void spmv_velocity(const DOp<T>& op, const V* __restr
 }
 
 // (B u) over one share of a pressure row's slots.
-template <typename T, typename V, int DIM, int kUS>
+template <typename T, typename V, int DIM, int kUS, bool EXACT>
 __device__ __forceinline__ V spmv_pressure(const DOp<T>& op, const V* __restrict__ x, int64_t q,
                                            int part, int parts) {
   const int64_t n2 = op.n2;
@@ -213,7 +217,7 @@ __device__ __forceinline__ V spmv_pressure(const DOp<T>& op, const V* __restrict
 #pragma unroll
       for (int u = 0; u < kUS; ++u) {
         if (skip_padding<V>() && k + u >= hi) break;
-        if (is_padding(bv[u][0])) continue;
+        if (left_out<EXACT>(bv[u][0])) continue;
 #pragma unroll
         for (int c = 0; c < DIM; ++c) acc += bv[u][c] * g[u][c];
       }
@@ -222,7 +226,7 @@ __device__ __forceinline__ V spmv_pressure(const DOp<T>& op, const V* __restrict
   return acc;
 }
 
-template <typename T, typename V, int DIM, int kUS>
+template <typename T, typename V, int DIM, int kUS, bool EXACT>
 __global__ void __launch_bounds__(256) k_spmv_full(DOp<T> op, JVec<const V> xv,
                                                    const V* __restrict__ b, JVec<V> yv,
                                                    int resid, SegSkip sku, SegSkip skp,
@@ -239,7 +243,7 @@ __global__ void __launch_bounds__(256) k_spmv_full(DOp<T> op, JVec<const V> xv,
     V acc[DIM];
 #pragma unroll
     for (int c = 0; c < DIM; ++c) acc[c] = V(0);
-    spmv_velocity<T, V, DIM, kUS>(op, x, row, 0, 1, acc);
+    spmv_velocity<T, V, DIM, kUS, EXACT>(op, x, row, 0, 1, acc);
 #pragma unroll
     for (int c = 0; c < DIM; ++c) {
       const int64_t r = c * n2 + row;
@@ -248,7 +252,7 @@ __global__ void __launch_bounds__(256) k_spmv_full(DOp<T> op, JVec<const V> xv,
   } else {
     const int64_t q = t;
     if (q >= nv || seg_skipped(skp, q)) return;
-    const V acc = spmv_pressure<T, V, DIM, kUS>(op, x, q, 0, 1);
+    const V acc = spmv_pressure<T, V, DIM, kUS, EXACT>(op, x, q, 0, 1);
     const int64_t r = DIM * n2 + q;
     const V v = acc + (V)op.diagp[q] * x[r];
     y[r] = resid ? b[r] - v : v;
@@ -258,7 +262,7 @@ __global__ void __launch_bounds__(256) k_spmv_full(DOp<T> op, JVec<const V> xv,
 // The same with a block per slice of 32 rows, whose W warps take a share of
 // the slots each (pressure slices first); a warp per component adds the
 // shares and finishes the rows.
-template <typename T, typename V, int DIM, int W, int kUS>
+template <typename T, typename V, int DIM, int W, int kUS, bool EXACT>
 __global__ void __launch_bounds__(32 * W) k_spmv_split(DOp<T> op, JVec<const V> xv,
                                                        const V* __restrict__ b, JVec<V> yv,
                                                        int resid, SegSkip sku, SegSkip skp,
@@ -278,8 +282,8 @@ __global__ void __launch_bounds__(32 * W) k_spmv_split(DOp<T> op, JVec<const V> 
 #pragma unroll
   for (int c = 0; c < DIM; ++c) acc[c] = V(0);
   if (act) {
-    if (pres) acc[0] = spmv_pressure<T, V, DIM, kUS>(op, x, row, w, W);
-    else spmv_velocity<T, V, DIM, kUS>(op, x, row, w, W, acc);
+    if (pres) acc[0] = spmv_pressure<T, V, DIM, kUS, EXACT>(op, x, row, w, W);
+    else spmv_velocity<T, V, DIM, kUS, EXACT>(op, x, row, w, W, acc);
   }
   // the finishing warps' own operands, before the shares are awaited
   const bool fin = act && w < (pres ? 1 : DIM);
@@ -1443,7 +1447,7 @@ inline unsigned grid_stride_blocks(int64_t n) {
 
 template <typename T, typename V>
 void launch_spmv_full(const DOp<T>& op, JVec<const V> x, const V* b, JVec<V> y, int resid,
-                      const int* skip, cudaStream_t s, bool seg) {
+                      const int* skip, cudaStream_t s, bool seg, bool exact) {
   const int64_t threads = ((op.nv + 31) & ~(int64_t)31) + op.n2;
   const SegSkip su = seg ? op.skip_u : SegSkip{}, sp = seg ? op.skip_p : SegSkip{};
   // slots per group: the schedule's, else 6 in FP32 and 4 in FP64 (FP64
@@ -1451,14 +1455,21 @@ void launch_spmv_full(const DOp<T>& op, JVec<const V> x, const V* b, JVec<V> y, 
   const int g = op.group ? op.group : (std::is_same<V, float>::value ? kUSpmv : kU);
   constexpr bool f32 = std::is_same<V, float>::value;
   const int share = op.group ? 1 : share_spmv(sizeof(V), op.dim, op.n2);
-#define FS_SPMVS(D, W)                                                                     \
-  launch_k(k_spmv_split<T, V, D, W, f32 ? 8 : 4>,                                          \
+#define FS_SPMVS(D, W)                                                                       \
+  launch_k(!f32 && exact ? k_spmv_split<T, V, D, W, f32 ? 8 : 4, !f32>                       \
+                         : k_spmv_split<T, V, D, W, f32 ? 8 : 4, false>,                     \
            (unsigned)((op.nv + 31) / 32 + (op.n2 + 31) / 32), 32 * W, 0, s, op, x, b, y, resid, \
            su, sp, skip)
 #define FS_SPMV(D, G) \
-  launch_k(k_spmv_full<T, V, D, G>, blocks_for(threads), 256, 0, s, op, x, b, y, resid, su, sp, \
-           skip)
-  if (share > 1) {
+  launch_k(k_spmv_full<T, V, D, G, false>, blocks_for(threads), 256, 0, s, op, x, b, y, resid, \
+           su, sp, skip)
+#define FS_SPMVX(D) \
+  launch_k(k_spmv_full<T, V, D, kU, !f32>, blocks_for(threads), 256, 0, s, op, x, b, y, resid, \
+           su, sp, skip)
+  if (!f32 && exact && share == 1) {  // (the depth is a matter of timing only)
+    if (op.dim == 2) FS_SPMVX(2);
+    else FS_SPMVX(3);
+  } else if (share > 1) {
     if (op.dim == 2) {
       if (share == 8) FS_SPMVS(2, 8);
       else FS_SPMVS(2, 4);
@@ -1476,14 +1487,16 @@ void launch_spmv_full(const DOp<T>& op, JVec<const V> x, const V* b, JVec<V> y, 
     else FS_SPMV(3, 4);
   }
 #undef FS_SPMVS
+#undef FS_SPMVX
 #undef FS_SPMV
   count_launches(1);
 }
 template void launch_spmv_full<double, double>(const DOp<double>&, JVec<const double>,
                                                const double*, JVec<double>, int, const int*,
-                                               cudaStream_t, bool);
+                                               cudaStream_t, bool, bool);
 template void launch_spmv_full<float, float>(const DOp<float>&, JVec<const float>, const float*,
-                                             JVec<float>, int, const int*, cudaStream_t, bool);
+                                             JVec<float>, int, const int*, cudaStream_t, bool,
+                                             bool);
 
 void launch_csr_to_sell(const DSell<double>& L, const int32_t* rp, const int32_t* ci,
                         const double* in, double* out64, float* out32, cudaStream_t s) {
