@@ -246,7 +246,11 @@ void fs_default_solve_opts(fs_solve_opts* opts);
  * x (device, FP64, n_dof) holds the initial guess and receives the solution;
  * NULL means the problem's state vector.  Synchronises.  stats may be NULL.
  * Returns FS_ERR_NOT_CONVERGED (with the best iterate kept) when max_iter or
- * max_refine is reached first, FS_ERR_NUMERIC on NaN/Inf. */
+ * max_refine is reached first, FS_ERR_NUMERIC on NaN/Inf, FS_ERR_TIMEOUT when
+ * a wait inside a kernel has not ended after one second (the blocks of the
+ * orthogonalisation kernel meet at barriers; the iterate is then undefined,
+ * and the problem can be solved again).  fs_step, fs_step_picard,
+ * fs_solve_steady and the server report the status of their solves. */
 int fs_solve(fs_problem* prob, const fs_solve_opts* opts, double* x,
              fs_solve_stats* stats);
 
@@ -322,7 +326,9 @@ int fs_solve_steady(fs_problem* prob, const fs_solve_opts* opts, double nl_tol,
  * positive definite once their boundary unknowns are eliminated; each is
  * solved in FP64 by Jacobi-preconditioned conjugate gradients to a relative
  * residual of rtol (checked every 8 iterations; FS_ERR_NOT_CONVERGED when
- * the true residual is above 100 rtol after max_iter iterations), whatever
+ * the true residual is above 100 rtol after max_iter iterations,
+ * FS_ERR_TIMEOUT when a wait inside the solve's one kernel has not ended after
+ * one second), whatever
  * the problem's precision.  Needs a single problem with Dirichlet velocity on
  * the whole boundary and the pressure pin (FS_ERR_UNSUPPORTED otherwise).
  * per_step (host, nsteps entries, may be NULL).  Synchronises. */

@@ -1308,7 +1308,10 @@ void finish_solve(fs_problem* P) {
   c.rc = FS_OK;
   for (int s = 0; s < P->nseg; ++s)
     if (c.status[s] != FS_OK && c.rc == FS_OK) c.rc = c.status[s];
-  if (c.rc != FS_OK) set_error("the solve did not reach rtol in every instance");
+  if (c.rc == FS_ERR_TIMEOUT)
+    set_error("a wait inside a solver kernel did not end within a second");
+  else if (c.rc != FS_OK)
+    set_error("the solve did not reach rtol in every instance");
   c.phase = PH_DONE;
 }
 
@@ -2564,7 +2567,10 @@ static int ipcs_cg(fs_problem* P, int which, const double* vals, const double* s
     FS_CUDA(cudaStreamSynchronize(s));
     *iters = c.iters;
     *relres = c.bb > 0 ? std::sqrt(c.rr / c.bb) : std::sqrt(c.rr);
-    if (c.bad) return FS_ERR_TIMEOUT;
+    if (c.bad) {
+      set_error("a wait inside the CG kernel did not end within a second");
+      return FS_ERR_TIMEOUT;
+    }
     if (!std::isfinite(*relres)) return FS_ERR_NUMERIC;
     return *relres <= 100.0 * rtol ? FS_OK : FS_ERR_NOT_CONVERGED;
   }

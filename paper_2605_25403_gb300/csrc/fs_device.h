@@ -29,8 +29,46 @@ void count_launches(int64_t n);
 // problem's schedule by the API entry points.
 bool launch_overlap();
 
+// Limit of a wait inside a kernel: one second.  A kernel whose wait runs out
+// marks its result and returns, and the call reports FS_ERR_TIMEOUT.
+constexpr uint64_t kWaitNs = 1000000000ull;
+
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+__device__ __forceinline__ uint64_t now_ns() {
+  uint64_t t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+// All blocks of a cooperative launch (which guarantees that they are resident
+// together) arrive before any leaves; false in every thread when the wait has
+// not ended after `limit` ns.  target counts the arrivals since the counter's
+// reset, modulo 2^32; ok: a word of shared memory.
+__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned target, uint64_t limit,
+                                             int* ok) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    *ok = 1;
+    if (gridDim.x > 1) {
+      __threadfence();
+      atomicAdd(bar, 1u);
+      const uint64_t t0 = now_ns();
+      unsigned v;
+      while (true) {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+        if ((int)(v - target) >= 0) break;
+        if (now_ns() - t0 >= limit) {
+          *ok = 0;
+          break;
+        }
+      }
+    }
+  }
+  __syncthreads();
+  return *ok != 0;
+}
 #endif
 
 template <typename... KArgs, typename... Args>
@@ -600,7 +638,6 @@ struct KCtl {
                            // arrivals, and their count before the launch
   uint64_t wait_ns;        // limit of each of that kernel's waits
 };
-constexpr uint64_t kWaitNs = 1000000000ull;  // one second
 
 template <typename V>
 void launch_seg_norm(const V* x, const TileList& tl, SegState* st, double* partial,

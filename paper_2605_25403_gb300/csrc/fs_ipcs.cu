@@ -398,44 +398,12 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_scalars(const double* part, i
 // vectors are walked flat, with the same thread on the same entries in every
 // phase.
 // ---------------------------------------------------------------------------
-constexpr uint64_t kCgWaitNs = 1000000000ull;  // one second per barrier
-
 struct CgShared {
   double sh[3][16];
   double sum[3];
   double post;
   int ok;
 };
-
-__device__ __forceinline__ uint64_t cg_clock() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-// All blocks arrive before any leaves; false after a second.
-__device__ bool cg_barrier(CgCtl* ctl, unsigned target, CgShared& S) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    S.ok = 1;
-    if (gridDim.x > 1) {
-      __threadfence();
-      atomicAdd(&ctl->bar, 1u);
-      const uint64_t t0 = cg_clock();
-      unsigned v;
-      while (true) {
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&ctl->bar) : "memory");
-        if ((int)(v - target) >= 0) break;
-        if (cg_clock() - t0 > kCgWaitNs) {
-          S.ok = 0;
-          break;
-        }
-      }
-    }
-  }
-  __syncthreads();
-  return S.ok != 0;
-}
 
 // The grid's sums of NS values, to S.sum: a block's own to part, a barrier,
 // then the partials in a fixed order.  An FP64 addition of a warp takes 64
@@ -446,7 +414,7 @@ __device__ bool cg_barrier(CgCtl* ctl, unsigned target, CgShared& S) {
 // additions, which every warp of the block would run.
 template <int NS, int LN, typename F>
 __device__ bool cg_grid_sum(double (&v)[NS], bool busy, double* part, CgCtl* ctl,
-                            unsigned target, CgShared& S, F post) {
+                            unsigned target, uint64_t limit, CgShared& S, F post) {
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   if (busy) {
 #pragma unroll
@@ -465,7 +433,7 @@ __device__ bool cg_grid_sum(double (&v)[NS], bool busy, double* part, CgCtl* ctl
       for (int u = 0; u < 4; ++u) t[u] += S.sh[threadIdx.x][i + u];  // nw is a multiple of 4
     part[NS * blockIdx.x + threadIdx.x] = (t[0] + t[1]) + (t[2] + t[3]);
   }
-  if (!cg_barrier(ctl, target, S)) return false;
+  if (!grid_barrier(&ctl->bar, target, limit, &S.ok)) return false;
   if (w < NS) {
     const int G = gridDim.x;
     double t[4] = {0, 0, 0, 0};
@@ -545,7 +513,7 @@ template <int DIM, int LN>
 __global__ void __launch_bounds__(512, 1)
     k_cg_solve(CgOp op, const double* rhs, double* x, const double* dinv, double* r, double* z,
                double* p, double* p2, double* q, double* part, CgCtl* ctl, double rtol,
-               int max_iter) {
+               int max_iter, uint64_t limit) {
   // small problems form the new direction at every neighbour (two buffers,
   // two barriers per iteration); where FP64 arithmetic counts it is a pass
   constexpr bool kFused = LN > 1;
@@ -559,6 +527,7 @@ __global__ void __launch_bounds__(512, 1)
   auto failed = [&]() {
     if (threadIdx.x == 0) ctl->bad = 1;
   };
+  auto meet = [&]() { return grid_barrier(&ctl->bar, ++bars * G, limit, &S.ok); };
   // eight lanes per row and one sweep: a lane keeps the first kHeld of its
   // entries (rows of up to 40) in registers through all iterations
   constexpr int kHeld = LN > 1 ? 5 : 1;
@@ -635,7 +604,7 @@ __global__ void __launch_bounds__(512, 1)
 #pragma unroll
       for (int c = 0; c < DIM; ++c) q[c * n + row] = s[c];
   });
-  if (!cg_barrier(ctl, ++bars * G, S)) return failed();
+  if (!meet()) return failed();
   double v[3] = {0, 0, 0};
   for (int64_t i = tid; i < N; i += nth) {
     const double b = rhs[i], ri = b - q[i], zi = dinv[i] * ri;
@@ -647,7 +616,7 @@ __global__ void __launch_bounds__(512, 1)
     v[2] += b * b;
   }
   const auto none = [](double) { return 0.0; };
-  if (!cg_grid_sum<3, 1>(v, busy, part0, ctl, ++bars * G, S, none)) return failed();
+  if (!cg_grid_sum<3, 1>(v, busy, part0, ctl, ++bars * G, limit, S, none)) return failed();
   double rz = S.sum[0], rr = S.sum[1], beta = 0.0;
   const double bb = S.sum[2], bn = sqrt(bb), tol2 = (rtol * bn) * (rtol * bn);
   int it = 0;
@@ -684,7 +653,7 @@ __global__ void __launch_bounds__(512, 1)
             }
         }
       });
-      if (!cg_grid_sum<1, LN>(pq, true, part1, ctl, ++bars * G, S,
+      if (!cg_grid_sum<1, LN>(pq, true, part1, ctl, ++bars * G, limit, S,
                               [rz](double t) { return t != 0.0 ? rz / t : 0.0; }))
         return failed();
       const double alpha = S.post;
@@ -697,7 +666,7 @@ __global__ void __launch_bounds__(512, 1)
         u[0] += ri * zi;
         u[1] += ri * ri;
       }
-      if (!cg_grid_sum<2, 1>(u, busy, part2, ctl, ++bars * G, S,
+      if (!cg_grid_sum<2, 1>(u, busy, part2, ctl, ++bars * G, limit, S,
                              [rz](double t) { return rz != 0.0 ? t / rz : 0.0; }))
         return failed();
       beta = S.post;
@@ -705,7 +674,7 @@ __global__ void __launch_bounds__(512, 1)
       rr = S.sum[1];
       if constexpr (!kFused) {
         for (int64_t i = tid; i < N; i += nth) pn[i] = z[i] + beta * pn[i];
-        if (!cg_barrier(ctl, ++bars * G, S)) return failed();
+        if (!meet()) return failed();
       }
     }
   }
@@ -722,7 +691,7 @@ __global__ void __launch_bounds__(512, 1)
       }
   });
   // (part1: without an iteration, blocks may still be reading part0)
-  if (!cg_grid_sum<1, LN>(e, true, part1, ctl, ++bars * G, S, none)) return failed();
+  if (!cg_grid_sum<1, LN>(e, true, part1, ctl, ++bars * G, limit, S, none)) return failed();
   if (tid == 0) {
     ctl->iters = it;
     ctl->rr = S.sum[0];
@@ -867,7 +836,8 @@ void launch_cg_solve(const DMesh& m, int which, const CgOp& op, const double* rh
   cfg.attrs = at;
   cfg.numAttrs = 1;
   auto go = [&](auto k) {
-    cudaLaunchKernelEx(&cfg, k, op, rhs, x, dinv, r, z, p, p2, q, part, ctl, rtol, max_iter);
+    cudaLaunchKernelEx(&cfg, k, op, rhs, x, dinv, r, z, p, p2, q, part, ctl, rtol, max_iter,
+                       kWaitNs);
   };
   if (which == 1) go(wide ? k_cg_solve<1, 8> : k_cg_solve<1, 1>);
   else if (m.dim == 2) go(wide ? k_cg_solve<2, 8> : k_cg_solve<2, 1>);

@@ -1609,7 +1609,6 @@ template void launch_precond<float>(const DOp<float>&, const DHier<float>&,
 namespace {
 
 constexpr int kFlowThreads = 512;
-constexpr uint64_t kFlowWaitNs = 1000000000ull;  // one second per wait
 
 enum { FL_LOAD_P = 0, FL_MG, FL_RESTRICT, FL_PROLONG, FL_DENSE, FL_PREC_P, FL_BT_ADD };
 
@@ -1657,11 +1656,6 @@ __device__ __forceinline__ unsigned flow_ld_acquire(const unsigned* p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
-}
-__device__ __forceinline__ uint64_t flow_clock_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
 }
 
 // Chebyshev pass over rows [r0, r1) of one hierarchy (NC real components
@@ -1827,9 +1821,9 @@ __global__ void __launch_bounds__(kFlowThreads, 2) k_prec_flow(FlowArgs<T> a) {
         const int64_t q = (int64_t)(it.phase - 1) * nseg + it.seg;
         const unsigned need = (unsigned)a.f.need[q];
         if (flow_ld_acquire(a.f.cnt + q) < need) {
-          const uint64_t t0 = flow_clock_ns();
+          const uint64_t t0 = now_ns();
           while (flow_ld_acquire(a.f.cnt + q) < need) {
-            if (flow_clock_ns() - t0 > kFlowWaitNs) {
+            if (now_ns() - t0 > kWaitNs) {
               // give up: the item runs on stale data and the solve reports it
               if (a.flag) a.flag[it.seg].bad = 2;
               break;

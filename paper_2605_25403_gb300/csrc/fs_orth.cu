@@ -74,12 +74,6 @@ __device__ __forceinline__ V warp_sum(V v) {
   return v;
 }
 
-__device__ __forceinline__ uint64_t now_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
 __device__ __forceinline__ void main_sync() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
 
 // 1 / sqrt(x) in FP64: the FP32 value and two Newton steps (relative error
@@ -91,32 +85,6 @@ __device__ __forceinline__ double inv_sqrt(double x) {
   const double h = 0.5 * x;
   y = y * (1.5 - h * y * y);
   return y * (1.5 - h * y * y);
-}
-
-// All blocks of the (cooperative) launch arrive before any leaves; false in
-// every thread when the wait has not ended after `limit` ns.  target counts
-// the arrivals since the barrier's reset, modulo 2^32.
-__device__ bool orth_barrier(KCtl* ctl, unsigned target, uint64_t limit, int* ok) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    *ok = 1;
-    if (gridDim.x > 1) {
-      __threadfence();
-      atomicAdd(&ctl->bar, 1u);
-      const uint64_t t0 = now_ns();
-      unsigned v;
-      while (true) {
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&ctl->bar) : "memory");
-        if ((int)(v - target) >= 0) break;
-        if (now_ns() - t0 >= limit) {
-          *ok = 0;
-          break;
-        }
-      }
-    }
-  }
-  __syncthreads();
-  return *ok != 0;
 }
 
 // A wait ran out: the cycle of every segment ends and the solve reports it
@@ -622,7 +590,7 @@ __global__ void __launch_bounds__(kOneThreads, 1)
   unsigned bars = 0;
   if (mode < ORTH_DOT) {
     bars += 1;
-    if (!orth_barrier(ctl, base + bars * gridDim.x, limit, &sh.ok)) {
+    if (!grid_barrier(&ctl->bar, base + bars * gridDim.x, limit, &sh.ok)) {
       if (tid == 0) orth_give_up(st, ctl, 1, cond);
       return;
     }
@@ -661,7 +629,7 @@ __global__ void __launch_bounds__(kOneThreads, 1)
     // second pass: every block took the same decision
     if (redo) {
       bars += 1;
-      if (!orth_barrier(ctl, base + bars * gridDim.x, limit, &sh.ok)) {
+      if (!grid_barrier(&ctl->bar, base + bars * gridDim.x, limit, &sh.ok)) {
         if (tid == 0) orth_give_up(st, ctl, 1, cond);
         return;
       }
@@ -998,7 +966,7 @@ __global__ void __launch_bounds__(kManyThreads, 1)
   unsigned bars = 0;
   auto meet = [&]() {
     bars += 1;
-    if (orth_barrier(ctl, base + bars * G, limit, &sh.ok)) return true;
+    if (grid_barrier(&ctl->bar, base + bars * G, limit, &sh.ok)) return true;
     if (tid == 0) orth_give_up(st, ctl, nseg, cond);
     land();
     return false;
