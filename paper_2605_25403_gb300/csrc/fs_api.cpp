@@ -2984,7 +2984,8 @@ int fs_autotune(fs_problem* P, int reps, fs_tune_report* report) {
   }
   if (!P->assembled) FS_TRY(assemble_impl(P, P->t + P->desc.dt));
   const int64_t cand[4] = {0, 4096, 16384, 65536};
-  const int sgroups[3] = {0, 4, 6}, pgroups[3] = {4, 6, 8};
+  // (group 0 alone shares rows among warps on small problems)
+  const int sgroups[3] = {0, 4, 6}, pgroups[4] = {0, 4, 6, 8};
   fs_tune_report r{};
   r.best = P->sched;
   FS_TRY(time_precond(P, reps, P->sched.persistent_precond, &r.default_ms));
@@ -3054,6 +3055,7 @@ int fs_autotune(fs_problem* P, int reps, fs_tune_report* report) {
   }
   // the SpMV: group depths, with the preconditioner's choice in place
   for (int g : pgroups) {
+    if (g == base.spmv_group) continue;  // timed as the default
     fs_schedule sc = r.best;
     sc.spmv_group = g;
     apply(sc);
