@@ -217,6 +217,7 @@ struct fs_problem {
   // both precisions)
   DSell<double> lA, lB, lBT;  // their layouts (no values)
   int64_t sA_slots = 0;       // value slots of lA
+  double op_index_bytes = 0;  // offsets and columns the product reads
   double *sA64 = nullptr, *sB64 = nullptr, *sBT64 = nullptr;
   // FP32 data (precision mode)
   float *sA32 = nullptr, *sB32 = nullptr, *sBT32 = nullptr, *diagp32 = nullptr;
@@ -467,6 +468,19 @@ std::vector<T> sell_values(const HostCsr& H, const SellLayout& L, const double* 
   return v;
 }
 
+// Bytes of offsets and columns that a pass over the rows reads: per slice an
+// offset (layouts of several widths), and 8 bytes per slot where the columns
+// are runs, else 4 per entry.
+double index_bytes(const HostCsr& H, const SellLayout& L) {
+  double b = L.width ? 0.0 : 8.0 * L.off.size();
+  for (int64_t sl = 0; sl < (int64_t)L.split.size(); ++sl) {
+    const int64_t r0 = 32 * sl, r1 = std::min(H.nrow, r0 + 32);
+    b += L.split[sl] > 0 ? 8.0 * ((L.off[sl + 1] - L.off[sl]) / 32)
+                         : 4.0 * (H.rowptr[r1] - H.rowptr[r0]);
+  }
+  return b;
+}
+
 // The layout's arrays on the device (values set by the caller).
 template <typename T>
 int upload_layout(fs_problem* P, const HostCsr& H, const SellLayout& L, DSell<T>& d) {
@@ -491,8 +505,9 @@ int upload_layout(fs_problem* P, const HostCsr& H, const SellLayout& L, DSell<T>
 
 template <typename T>
 int upload_sell(fs_problem* P, const HostCsr& H, DSell<T>& d, double uniform_slack,
-                const Owners* owner) {
+                const Owners* owner, double* index) {
   const SellLayout L = sell_layout(H, uniform_slack, owner, owner);
+  if (index) *index = index_bytes(H, L);
   FS_TRY(upload_layout(P, H, L, d));
   std::vector<T> v = sell_values<T>(H, L, H.val.data(), 1);
   T* dv;
@@ -611,7 +626,8 @@ int upload_hierarchy(fs_problem* P, const UnionHierarchy& U, int nc, DHier<T>& D
                   (int32_t)i);
       owner.finish();
     }
-    FS_TRY(upload_sell<T>(P, hl.A, dl.A, 0.15, batch ? &owner : nullptr));
+    FS_TRY(upload_sell<T>(P, hl.A, dl.A, 0.15, batch ? &owner : nullptr,
+                          l == 0 ? &D.fine_index_bytes : nullptr));
     if (l + 1 < D.nlev) {
       FS_TRY(upload_csr<T>(P, hl.P, dl.P));
       FS_TRY(upload_csr<T>(P, hl.R, dl.R));
@@ -2107,6 +2123,7 @@ int fs_problem_create_batch(fs_mesh* mesh, const fs_problem_desc* descs, int cou
     FS_TRY(upload_layout(P.get(), me.B, LB, P->lB));
     FS_TRY(upload_layout(P.get(), me.BT, LBT, P->lBT));
     P->sA_slots = LA.off.back();
+    P->op_index_bytes = index_bytes(me.A, LA) + index_bytes(me.B, LB) + index_bytes(me.BT, LBT);
     FS_TRY(P->alloc(&P->sA64, LA.off.back()));
     FS_CUDA(cudaMemsetAsync(P->sA64, 0, sizeof(double) * LA.off.back(), s));
     FS_TRY(P->upload(&P->sB64, sell_values<double>(me.B, LB, Bh.data(), dim)));
@@ -2789,8 +2806,8 @@ int fs_profile_kernel(fs_problem* P, int kernel, int reps, double* avg_ms, doubl
     case FS_KERNEL_SPMV_FP64: {
       const bool use32 = f32 && kernel == FS_KERNEL_SPMV;
       const double sz = use32 ? 4.0 : 8.0;
-      bytes = nnzA * (4 + sz) + nnzBT * (4 + d * sz) + nnzB * (4 + d * sz) +
-              4.0 * (2 * (P->n2 + 1) + (P->nv + 1)) + P->nv * sz + 2.0 * P->ndof * sz;
+      bytes = (nnzA + d * nnzBT + d * nnzB) * sz + P->op_index_bytes + P->nv * sz +
+              2.0 * P->ndof * sz;
       if (use32) {
         auto& pr = P->p32;
         launch = [P, &pr]() {
@@ -2807,7 +2824,8 @@ int fs_profile_kernel(fs_problem* P, int kernel, int reps, double* avg_ms, doubl
     }
     case FS_KERNEL_CHEB: {  // one fused Chebyshev step on the finest velocity level
       const int64_t n = P->n2;
-      bytes = nnzA * (4 + s) + 4.0 * (n + 1) + n * s + 5.0 * d * n * s;
+      const double index = f32 ? P->p32.HA.fine_index_bytes : P->p64.HA.fine_index_bytes;
+      bytes = nnzA * s + index + n * s + 5.0 * d * n * s;
       if (f32) {
         const DHier<float> H = without_skip(P->p32.HA);
         launch = [P, H, d]() { launch_cheb_step<float>(H, d, P->stream); };

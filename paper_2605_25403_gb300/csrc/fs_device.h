@@ -373,6 +373,7 @@ struct DHier {
   // first level run by the fused cluster kernel (-1: none), its cluster size
   int tail = -1;
   int tail_cluster = 8;
+  double fine_index_bytes = 0;  // offsets and columns a pass over level 0 reads
   // a copy of this struct in device memory (read by the coarse kernels)
   const DHier<T>* dev = nullptr;
 };
