@@ -70,8 +70,9 @@ def parse(argv=None):
                         "CUDA graphs (for per-kernel profilers, which cannot see kernels inside "
                         "graphs with conditional nodes)")
     p.add_argument("--roofline-kernel", default="cgs_upd", choices=sorted(KERNELS),
-                   help="kernel of the roofline line: the largest single kernel of the "
-                        "channel step's ncu launch list (the CGS2 update pass)")
+                   help="kernel of the roofline line; cgs_upd is the orthogonalisation's update "
+                        "pass with its re-dots, which a step takes only when its first pass "
+                        "cancels most of the vector (orth: the launch an ordinary step runs)")
     p.add_argument("--batch-steps", type=int, default=20,
                    help="timed steps of the 96-instance batched workload (0: skip)")
     p.add_argument("--cube-steps", type=int, default=10,
@@ -100,7 +101,14 @@ KERNELS = {
     "cgs_dot": ("FS_KERNEL_CGS_DOT", "k_orth_one/k_orth_many, dot pass alone (V^T w and V^T v_j, j = 15)"),
     "cgs_upd": ("FS_KERNEL_CGS_UPD", "k_orth_one/k_orth_many, update pass with the re-dots alone (j = 15)"),
     "cgs_fin": ("FS_KERNEL_CGS_FIN", "k_orth_one/k_orth_many, second pass alone (j = 15)"),
+    "orth": ("FS_KERNEL_ORTH", "k_orth_one/k_orth_many, dot pass, barrier and update in one launch "
+                               "(j = 15, as an ordinary step runs it, without the Givens step)"),
 }
+
+# names of the kernels' records in profiles/traffic.txt where they differ: the
+# operator kernels were captured with a column index per entry and again with
+# the columns as runs
+TRAFFIC = {"cheb": "cheb_runs", "spmv": "spmv_runs"}
 
 
 SMOOTHER_DEGREES = ((2, 2), (1, 2), (2, 1), (1, 1))
@@ -654,7 +662,7 @@ def main():
                 "frac": achieved / peak, "peak_source": peak_kind, "kernel": KERNELS[kname][1],
                 "timing": "L2-cold, each launch after a read of twice the L2 size, CUDA events "
                           "on the problem's stream",
-                "traffic": traffic_from_profiles(kname, wl.name)}
+                "traffic": traffic_from_profiles(TRAFFIC.get(kname, kname), wl.name)}
 
     # ---- CPU baseline: the oracle on a bounded sample ---------------------
     cpu = None

@@ -592,6 +592,10 @@ enum {
                                    norm): j + 3 sweeps                    */
   FS_KERNEL_CGS_FIN = 8,        /* its second pass alone (w -= V h2,
                                    normalise): j + 3 sweeps               */
+  FS_KERNEL_ORTH = 9,           /* one orthogonalisation as a step runs it when
+                                   its first pass suffices (dot pass, barrier,
+                                   update), without the Givens rotations:
+                                   2j + 5 sweeps                          */
   FS_PROFILE_COLD_L2 = 0x100    /* flag: L2-cold timing, see above        */
 };
 int64_t fs_launch_count(void);

@@ -2852,7 +2852,8 @@ int fs_profile_kernel(fs_problem* P, int kernel, int reps, double* avg_ms, doubl
     case FS_KERNEL_CGS:  // one CGS2 step of the Arnoldi process at j = m/2
     case FS_KERNEL_CGS_DOT:
     case FS_KERNEL_CGS_UPD:
-    case FS_KERNEL_CGS_FIN: {
+    case FS_KERNEL_CGS_FIN:
+    case FS_KERNEL_ORTH: {
       // Krylov scratch only (basis, cycle state): the next solve rebuilds it.
       // Step index j and active segments are set on the device first.
       auto prime = [P](auto& K, int* jout) -> int {
@@ -2883,7 +2884,10 @@ int fs_profile_kernel(fs_problem* P, int kernel, int reps, double* avg_ms, doubl
       // basis vectors each pass must touch, each counted once: dot reads
       // V[0..j] and w; update reads V[0..j] and w and writes w (its re-dot
       // reads V[0..j] again, which is not counted); final the same
-      const double sweeps = pass < 0 ? 3.0 * j + 8.0 : pass == 0 ? j + 2.0 : j + 3.0;
+      const double sweeps = pass < 0 ? 3.0 * j + 8.0
+                            : pass == 0 ? j + 2.0
+                            : pass == 3 ? 2.0 * j + 5.0
+                                        : j + 3.0;
       bytes = sweeps * (double)P->ndof * s;
       break;
     }

@@ -680,8 +680,8 @@ template <typename V>
 void launch_seg_orth(V* Vb, int64_t ld, const OrthPlan& P, SegState* st, KCtl* ctl,
                      cudaGraphConditionalHandle cond, cudaStream_t s);
 // For kernel timing, without the Givens step: the orthogonalisation with its
-// second pass always taken (pass < 0), or its dot pass (0), its update pass
-// with the re-dots (1) or its second pass (2) alone.
+// second pass always taken (pass < 0) or never (3), or its dot pass (0), its
+// update pass with the re-dots (1) or its second pass (2) alone.
 template <typename V>
 void launch_seg_orth_pass(V* Vb, int64_t ld, const OrthPlan& P, SegState* st, KCtl* ctl, int pass,
                           cudaStream_t s);

@@ -374,6 +374,14 @@ __device__ __forceinline__ void reduce_sums(OrthShared<V>& sh, const double* par
   __syncthreads();
 }
 
+// What a launch runs: a whole Arnoldi step with its Givens rotations, or
+// for timing the orthogonalisation alone, with both passes taken (ORTH_FULL),
+// with the first only (ORTH_ONCE), or one of its passes.
+enum { ORTH_STEP = 0, ORTH_FULL, ORTH_ONCE, ORTH_DOT, ORTH_UPD, ORTH_FIN };
+__device__ __forceinline__ bool second_pass(int mode, double hn2, double ww) {
+  return mode == ORTH_STEP ? hn2 < kRedo * ww : mode != ORTH_ONCE;
+}
+
 // From the sums of the dot pass (sh.sum) and E: c = E a, then h, hn and the
 // decision on a second pass (whole block; sh.hcol, sh.f and sh.redo are
 // valid after the caller's next barrier).  Row j of E goes to S when store.
@@ -381,7 +389,7 @@ __device__ __forceinline__ void reduce_sums(OrthShared<V>& sh, const double* par
 // whose additions over the lanes would cost most of it, a lane takes a row
 // and four warps (one per quarter SM) eight columns each.
 template <typename V>
-__device__ __forceinline__ void first_column(OrthShared<V>& sh, int j, bool force, SegState& S,
+__device__ __forceinline__ void first_column(OrthShared<V>& sh, int j, int mode, SegState& S,
                                              bool store) {
   constexpr bool f32 = sizeof(V) == 4;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nvec = j + 1;
@@ -420,7 +428,7 @@ __device__ __forceinline__ void first_column(OrthShared<V>& sh, int j, bool forc
     if (lane == 0) {
       sh.hcol[nvec] = hn2 > 0.0 ? hn2 * f : isfinite(hn2) ? 0.0 : hn2;
       sh.f = f;
-      sh.redo = (force || hn2 < kRedo * ww) ? 1 : 0;
+      sh.redo = second_pass(mode, hn2, ww) ? 1 : 0;
     }
   }
 }
@@ -538,11 +546,6 @@ __device__ void end_arnoldi_step(KCtl* ctl, int j, int m, cudaGraphConditionalHa
   if (cond) cudaGraphSetConditional(cond, (!all && j + 1 < m) ? 1u : 0u);
 }
 
-// What a launch runs: a whole Arnoldi step with its Givens rotations, or
-// for timing the orthogonalisation alone with both passes taken (ORTH_FULL)
-// or one of its passes.
-enum { ORTH_STEP = 0, ORTH_FULL, ORTH_DOT, ORTH_UPD, ORTH_FIN };
-
 // ---------------------------------------------------------------------------
 // One segment, share entries per block from block b's b share on.  (Keeping
 // the block's share of the basis in shared memory between the passes, by bulk
@@ -600,7 +603,7 @@ __global__ void __launch_bounds__(kOneThreads, 1)
   if (mode != ORTH_FIN) {
     reduce_sums(sh, part1, n1, gridDim.x);
     clear_sums(sh, n2);
-    first_column(sh, j, mode != ORTH_STEP, S, owner && mode == ORTH_STEP);
+    first_column(sh, j, mode, S, owner && mode == ORTH_STEP);
     __syncthreads();
     redo = sh.redo != 0;
     if (!work && lane <= j) 
@@ -995,7 +998,7 @@ __global__ void __launch_bounds__(kManyThreads, 1)
       if (givens && mode != ORTH_STEP)
         for (int i = 0; i < 33; ++i) sh.E[i * 32 + lane] = V(0);
       reduce_sums(sh, part1 + (int64_t)P.seg_slot[2 * s] * 64, n1, P.seg_slot[2 * s + 1]);
-      first_column(sh, j, mode != ORTH_STEP, S, mode == ORTH_STEP);
+      first_column(sh, j, mode, S, mode == ORTH_STEP);
       __syncthreads();
       if (warp == 0) {
         if (lane <= nvec) S.h2[lane] = sh.hcol[lane];
@@ -1083,7 +1086,7 @@ __global__ void __launch_bounds__(kManyThreads, 1)
     if (mode == ORTH_UPD) return land();
   }
   // ---- second pass ----------------------------------------------------------
-  const int nredo = mode == ORTH_STEP ? *(volatile int*)&ctl->nredo : 1;
+  const int nredo = mode <= ORTH_ONCE ? *(volatile int*)&ctl->nredo : 1;
   if (nredo > 0) {
     if (mode != ORTH_FIN && !meet()) return;
     for (int s = blockIdx.x; s < nseg; s += G) {
@@ -1192,7 +1195,8 @@ template void launch_seg_orth<float>(float*, int64_t, const OrthPlan&, SegState*
 template <typename V>
 void launch_seg_orth_pass(V* Vb, int64_t ld, const OrthPlan& P, SegState* st, KCtl* ctl, int pass,
                           cudaStream_t s) {
-  const int mode = pass < 0 ? ORTH_FULL : pass == 0 ? ORTH_DOT : pass == 1 ? ORTH_UPD : ORTH_FIN;
+  constexpr int kMode[] = {ORTH_DOT, ORTH_UPD, ORTH_FIN, ORTH_ONCE};
+  const int mode = pass < 0 ? ORTH_FULL : kMode[pass];
   launch_orth(Vb, ld, P, st, ctl, 0, mode, s);
 }
 template void launch_seg_orth_pass<double>(double*, int64_t, const OrthPlan&, SegState*, KCtl*,

@@ -212,7 +212,7 @@ EXPORTED = ["fs_mesh_create", "fs_mesh_destroy", "fs_dof_map", "fs_problem_creat
             "fs_problem_sizes"]
 (FS_KERNEL_SPMV, FS_KERNEL_SPMV_FP64, FS_KERNEL_CHEB, FS_KERNEL_ASSEMBLE_CONV,
  FS_KERNEL_PRECOND, FS_KERNEL_CGS, FS_KERNEL_CGS_DOT, FS_KERNEL_CGS_UPD,
- FS_KERNEL_CGS_FIN) = range(9)
+ FS_KERNEL_CGS_FIN, FS_KERNEL_ORTH) = range(10)
 FS_PROFILE_COLD_L2 = 0x100
 
 

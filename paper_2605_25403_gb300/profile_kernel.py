@@ -24,7 +24,7 @@ def main(argv=None):
     p.add_argument("--workload", default="cube", choices=["channel", "cube", "unit_square"])
     p.add_argument("--kernel", default="cheb",
                    choices=["cheb", "spmv", "spmv_fp64", "assemble", "precond", "cgs",
-                            "cgs_dot", "cgs_upd", "cgs_fin"])
+                            "cgs_dot", "cgs_upd", "cgs_fin", "orth"])
     p.add_argument("--cold", action="store_true",
                    help="time each launch after the L2 was filled with other data")
     p.add_argument("--precision", default="fp32_refine", choices=["fp32_refine", "fp64"])
@@ -45,7 +45,7 @@ def main(argv=None):
            "spmv_fp64": fs.FS_KERNEL_SPMV_FP64, "assemble": fs.FS_KERNEL_ASSEMBLE_CONV,
            "precond": fs.FS_KERNEL_PRECOND, "cgs": fs.FS_KERNEL_CGS,
            "cgs_dot": fs.FS_KERNEL_CGS_DOT, "cgs_upd": fs.FS_KERNEL_CGS_UPD,
-           "cgs_fin": fs.FS_KERNEL_CGS_FIN}[a.kernel]
+           "cgs_fin": fs.FS_KERNEL_CGS_FIN, "orth": fs.FS_KERNEL_ORTH}[a.kernel]
     S = fs.Stepper.from_workload(wl, precision=prec)
     try:
         ms, by = fs.fs_profile_kernel(S.prob, kid, reps=a.reps, cold=a.cold)

@@ -37,3 +37,23 @@ def test_operator_bytes(fs, wl):
         assert 0 < index <= 0.4 * 4 * nnza
     finally:
         S.close()
+
+
+# one segment in one block's reach, streamed, and a batch
+@pytest.mark.parametrize("wls", [[W.unit_square(40)], [W.unit_square(290, nu=0.01, dt=1e-3)],
+                                 [W.unit_square(n, jitter=0.0) for n in (30, 7, 41)]],
+                         ids=["one", "streamed", "batch"])
+def test_orthogonalisation_as_a_step_runs_it(fs, wls):
+    S = fs.Stepper.from_workloads(wls, precision=fs.FS_PREC_FP32_REFINE) if len(wls) > 1 else \
+        fs.Stepper.from_workload(wls[0], precision=fs.FS_PREC_FP32_REFINE)
+    try:
+        fs.fs_step(S.prob, 1)
+        x0, t0 = S.state()
+        ms, by = fs.fs_profile_kernel(S.prob, fs.FS_KERNEL_ORTH, 20)
+        both = fs.fs_profile_kernel(S.prob, fs.FS_KERNEL_CGS, 20)[0]
+        assert by == (2 * 15 + 5) * S.info["n_dof"] * 4 and 0 < ms < both
+        x, t = S.state()
+        assert (x == x0).all() and t == t0
+        assert fs.fs_step(S.prob, 1)[0]["status"] == 0
+    finally:
+        S.close()
