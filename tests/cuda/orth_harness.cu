@@ -165,7 +165,7 @@ int step(const Case& c, const int64_t* seg0, const double* Vin, double* E, doubl
     const int32_t out[4] = {S.bad, S.done, S.act, S.k};
     std::copy(out, out + 4, seg_out + 4 * s);
   }
-  const int32_t out[4] = {k.j, k.all_done, k.nredo, (int32_t)(k.bar - k.bar_base)};
+  const int32_t out[4] = {k.j, k.all_done, k.nredo, (int32_t)k.bar};
   std::copy(out, out + 4, ctl_out);
   return 0;
 }

@@ -51,7 +51,7 @@ def step(lib, f32, case, V, E=None, state=None):
     """One step on the rows V (j + 2 of them): the new vector, per segment the
     Hessenberg column, the Gram correction, (bad, done, act, k), the rotation
     before this step's and the segments' records (a later step's `state`, which
-    then holds E); and (j, all_done, nredo, arrivals)."""
+    then holds E); and (j, all_done, nredo, barrier arrivals)."""
     c, seg0 = case
     V = np.ascontiguousarray(V, dtype=np.float64)
     assert V.shape == (c.j + 2, c.n)

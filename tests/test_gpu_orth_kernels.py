@@ -142,3 +142,48 @@ def test_rotation_takes_the_norm_of_the_stored_vector(lib, many, f32):
         want = s / c * float(norm)
         assert abs(rot[1] / rot[0] / want - 1) <= (9 * 6e-8 / np.sqrt(n / 128) if f32 else 3e-15)
     assert worst > (1e-7 if f32 else 1e-15)  # the norms were off
+
+
+def _check_segments(V, seg0, out, u, redo):
+    """Arnoldi relation, norm and orthogonality of every segment; a sum of up to
+    31 products of rows with entries rounded by u."""
+    j = len(V) - 2
+    for s, (a, b) in enumerate(zip(seg0[:-1], seg0[1:])):
+        Q, w, x, h = V[:j + 1, a:b], V[j + 1, a:b], out["w"][a:b], out["h"][s]
+        assert np.linalg.norm(h[:j + 1] @ Q + h[j + 1] * x - w) <= 60 * u
+        # one pass: the sums' rounding over hn; two: that of the second alone
+        grow = 1.0 if redo[s] else np.sqrt(1 / 0.01)
+        assert abs(np.linalg.norm(x) - 1) <= 20 * u * grow
+        assert np.abs(Q @ x).max() <= 20 * u * grow
+
+
+# the second pass: taken by a segment whose first cancels most of the vector,
+# in a batch by some segments and not by others, and by blocks with more pieces
+# than their list holds (three rounds of it)
+@pytest.mark.parametrize("f32", [False, True])
+@pytest.mark.parametrize("lens,piece,blocks,inside", [
+    ([1501], 0, 3, [1e-4]),
+    ([1501], 0, 1, [1e-6]),
+    ([3000], 256, 5, [1e-4]),
+    ([700, 301, 33, 2049, 64], 256, 6, [0.5, 1e-4, 0.3, 1e-5, 0.02]),
+    ([9000, 37, 8000, 2963], 4, 2, [0.5, 0.4, 1e-4, 0.3]),
+    ([9000, 37, 8000, 2963], 4, 2, [0.5, 0.4, 0.1, 0.3])],
+    ids=["one", "one_block", "streamed", "some", "rounds", "rounds_single_pass"])
+def test_second_pass(lib, lens, piece, blocks, inside, f32):
+    r = np.random.RandomState(5)
+    j = 9
+    ty = np.float32 if f32 else np.float64
+    case = H.many(lens, piece, blocks, j) if piece else \
+        H.one(lens[0], (-(-lens[0] // blocks) + 31) // 32 * 32, j)
+    V = np.concatenate([H.basis(r, j, n, inside=q) for n, q in zip(lens, inside)], axis=1)
+    V = V.astype(ty).astype(np.float64)
+    _, _, E = H.reference(V, case[1], ty)
+    out = H.step(lib, f32, case, V, E)
+    redo = [q < 0.01 for q in inside]
+    assert (out["seg"][:, 0] == 0).all() and out["ctl"][0] == j + 1 and out["ctl"][2] == 0
+    if piece:
+        assert out["seg"][:, 2].tolist() == [2 if q else 1 for q in redo]
+        assert out["ctl"][3] == case[0].blocks * (4 if any(redo) else 2)
+    else:
+        assert out["ctl"][3] == (2 * case[0].blocks if case[0].blocks > 1 else 0)
+    _check_segments(V, case[1], out, 6e-8 if f32 else 1.2e-16, redo)
