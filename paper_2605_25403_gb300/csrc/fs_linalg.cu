@@ -322,7 +322,10 @@ __global__ void k_csr_to_sell(DSell<double> L, const int32_t* __restrict__ rp,
     int32_t k = rp[r];
     for (int u = 0; u < R.w; ++u) {
       double v = -0.0;
-      if (k < e && ci[k] == col(u) + shift) v = in[k++] + 0.0;
+      if (k < e && ci[k] == col(u) + shift) {
+        v = in[k++];
+        if (left_out<true>(v)) v = 0.0;  // a zero entry is no padding
+      }
       out64[base + 32 * u] = v;
       if (out32) out32[base + 32 * u] = (float)v;
     }

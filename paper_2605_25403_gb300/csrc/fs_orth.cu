@@ -578,14 +578,14 @@ __global__ void __launch_bounds__(kOneThreads, 1)
   V* bv = Vb + start;
   V* vw = bv + (int64_t)nvec * ld;
   clear_sums(sh, n1);
-  if (!work && mode < ORTH_DOT)  // E, read while the dot pass runs
-    load_gram(sh.E, gram<V>(S), j);
   if (mode == ORTH_UPD && !work)
     for (int i = 0; i < 33; ++i) sh.E[i * 32 + lane] = V(0);
   __syncthreads();
   if (mode <= ORTH_DOT) {
     if (work)
       dot_piece<V, LE, NB, true>(bv, ld, nvec, vw, vw - ld, len, P.T, sh.wpart[warp]);
+    else if (mode < ORTH_DOT)
+      load_gram(sh.E, gram<V>(S), j);  // while the dot pass runs
     __syncthreads();
     store_sums(sh, part1 + (int64_t)blockIdx.x * 64, n1);
     if (mode == ORTH_DOT) return;
