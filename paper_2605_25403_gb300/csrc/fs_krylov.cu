@@ -173,8 +173,27 @@ __device__ __forceinline__ double widen(float z) {
   const unsigned b = __float_as_uint(z);
   return __hiloint2double((int)((b & 0x80000000u) | ((b & 0x7fffffffu) >> 3)), (int)(b << 29));
 }
-__device__ __forceinline__ bool finite_bits(float z) {
-  return (__float_as_uint(z) & 0x7f800000u) != 0x7f800000u;
+// The sum over the directions by conversion.  For FP32 directions that are not
+// all finite it is a call: inlined, the compiler would convert beside every
+// widened entry and select.
+template <typename V>
+__device__ __forceinline__ double sum_directions_impl(const V* __restrict__ z, int64_t n, int k,
+                                                      const double* y) {
+  double s[4] = {0, 0, 0, 0};
+  int c = 0;
+  for (; c + 4 <= k; c += 4) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) s[u] += y[c + u] * (double)z[(int64_t)(c + u) * n];
+  }
+  for (; c < k; ++c) s[0] += y[c] * (double)z[(int64_t)c * n];
+  return (s[0] + s[1]) + (s[2] + s[3]);
+}
+__device__ __forceinline__ double sum_directions(const double* z, int64_t n, int k,
+                                                 const double* y) {
+  return sum_directions_impl(z, n, k, y);
+}
+__device__ __noinline__ double sum_directions(const float* z, int64_t n, int k, const double* y) {
+  return sum_directions_impl(z, n, k, y);
 }
 
 // y = H(0:k,0:k)^-1 g(0:k) of the tile's segment, then x += Z y.
@@ -184,7 +203,11 @@ __device__ __forceinline__ bool finite_bits(float z) {
 // memory (one thread walking it through global memory took most of the
 // kernel's time on small vectors).  The sums over the directions run in FP64,
 // FP32 directions widened by their bits (unless one is not finite, or a
-// coefficient is 2^127 or more): FP64 arithmetic is what bounds the kernel.
+// coefficient is 2^127 or more): FP64 arithmetic is what bounds the kernel (109
+// us of FMAs on the 48^3 cube).  Per cycle on GB300, 24 directions or so: 78 ->
+// 32 us on the 512x96 channel, 418 -> 189 on the 48^3 cube, 209 -> 107 on the
+// batch of 96 squares, 48 -> 24 on the FP64 8^2 square (sums of FP32 pairs, 48
+// bits, took 35, 163 and 81 us).
 template <typename V, typename X>
 __global__ void __launch_bounds__(kKB) k_seg_update_x(const SegState* st, const KCtl* ctl,
                                                       const V* __restrict__ Z, int64_t n,
@@ -224,26 +247,35 @@ __global__ void __launch_bounds__(kKB) k_seg_update_x(const SegState* st, const 
   const bool bits = f32 && by_bits;
   for (int e = threadIdx.x; e < t.len; e += kKB) {
     const int64_t i = t.start + e;
-    // four directions at a time into separate sums (independent loads)
-    double s[4] = {0, 0, 0, 0};
-    int c = 0;
-    for (; c + 4 <= k; c += 4) {
-      V z[4];
+    double sum = 0.0;
+    bool done = false;
+    if constexpr (f32) {
+      if (bits) {
+        // four directions at a time into separate sums (independent loads)
+        double s[4] = {0, 0, 0, 0};
+        unsigned top = 0;  // largest exponent field
+        int c = 0;
+        for (; c + 4 <= k; c += 4) {
+          float z[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) z[u] = Z[(int64_t)(c + u) * n + i];
-      if constexpr (f32) {
-        if (bits && finite_bits(z[0]) && finite_bits(z[1]) && finite_bits(z[2]) &&
-            finite_bits(z[3])) {
+          for (int u = 0; u < 4; ++u) z[u] = Z[(int64_t)(c + u) * n + i];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) s[u] += ys[c + u] * widen(z[u]);
-          continue;
+          for (int u = 0; u < 4; ++u) {
+            top = max(top, __float_as_uint(z[u]) & 0x7f800000u);
+            s[u] += ys[c + u] * widen(z[u]);
+          }
         }
+        for (; c < k; ++c) {
+          const float z = Z[(int64_t)c * n + i];
+          top = max(top, __float_as_uint(z) & 0x7f800000u);
+          s[0] += ys[c] * widen(z);
+        }
+        sum = (s[0] + s[1]) + (s[2] + s[3]);
+        done = top != 0x7f800000u;  // all finite
       }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) s[u] += y[c + u] * (double)z[u];
     }
-    for (; c < k; ++c) s[0] += y[c] * (double)Z[(int64_t)c * n + i];
-    x[i] = (X)((double)x[i] + ((s[0] + s[1]) + (s[2] + s[3])));
+    if (!done) sum = sum_directions(Z + i, n, k, y);
+    x[i] = (X)((double)x[i] + sum);
   }
 }
 
