@@ -323,6 +323,7 @@ struct OrthShared {
   double wpart[kOrthWarps][64];  // a warp's sums
   double red[kOrthMain];
   double sum[64];
+  V vsum[64];  // the first reduction's in the vectors' type, e_j less its 1
   double hcol[kMaxRestart + 1];  // the Hessenberg column
   V E[32 * 33];
   V c[4][32];  // E a (FP64: in four shares of the columns)
@@ -347,10 +348,10 @@ __device__ __forceinline__ void store_sums(const OrthShared<V>& sh, double* slot
 }
 
 // sh.sum = the first ns sums added over count slots (64 apart), in a fixed
-// order (whole block).
+// order (whole block).  unit: the index of v_j . v_j among them (-1: none).
 template <typename V>
 __device__ __forceinline__ void reduce_sums(OrthShared<V>& sh, const double* part, int ns,
-                                            int count) {
+                                            int count, int unit) {
   const int tid = threadIdx.x;
   const int parts = kOrthMain / ns, g = tid / ns, s = tid - g * ns;
   if (g < parts) {
@@ -378,7 +379,9 @@ __device__ __forceinline__ void reduce_sums(OrthShared<V>& sh, const double* par
       for (int u = 0; u < 4; ++u)
         if (q + u < used) v[u] += sh.red[(q + u) * ns + tid];
     }
-    sh.sum[tid] = (v[0] + v[1]) + (v[2] + v[3]);
+    const double s = (v[0] + v[1]) + (v[2] + v[3]);
+    sh.sum[tid] = s;
+    if (unit >= 0) sh.vsum[tid] = (V)(tid == unit ? s - 1.0 : s);
   }
   __syncthreads();
 }
@@ -402,9 +405,9 @@ __device__ __forceinline__ void first_column(OrthShared<V>& sh, int j, int mode,
                                              bool store) {
   constexpr bool f32 = sizeof(V) == 4;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nvec = j + 1;
-  const V e = lane < nvec ? (V)(sh.sum[nvec + lane] - (lane == j ? 1.0 : 0.0)) : V(0);
+  const V e = lane < nvec ? sh.vsum[nvec + lane] : V(0);
   if (f32 && warp < kOrthWarps) {
-    const V a = lane < nvec ? (V)sh.sum[lane] : V(0);
+    const V a = lane < nvec ? sh.vsum[lane] : V(0);
     for (int i = warp; i < nvec; i += kOrthWarps) {
       // row i of E: E[i][k] for k < j, e_i in column j; row j is e
       const V ei = __shfl_sync(kFull, e, i);
@@ -417,7 +420,7 @@ __device__ __forceinline__ void first_column(OrthShared<V>& sh, int j, int mode,
     for (int k = 8 * warp; k < 8 * warp + 8 && k < nvec; ++k) {
       const V ek = __shfl_sync(kFull, e, k);
       const V r = lane == j ? ek : lane > j ? V(0) : k == j ? e : sh.E[lane * 33 + k];
-      s += r * (V)sh.sum[k];
+      s += r * sh.vsum[k];
     }
     sh.c[warp][lane] = s;
   } else if (warp >= kOrthWarps && store && lane < nvec) {
@@ -610,13 +613,13 @@ __global__ void __launch_bounds__(kOneThreads, 1)
   bool redo = true;
   V vsq = V(0);  // |v_lane|^2 - 1
   if (mode != ORTH_FIN) {
-    reduce_sums(sh, part1, n1, gridDim.x);
+    reduce_sums(sh, part1, n1, gridDim.x, nvec + j);
     clear_sums(sh, n2);
     first_column(sh, j, mode, S, owner && mode == ORTH_STEP);
     __syncthreads();
     redo = sh.redo != 0;
     if (!work && lane <= j)
-      vsq = lane < j ? sh.E[lane * 34] : (V)(sh.sum[nvec + j] - 1.0);
+      vsq = lane < j ? sh.E[lane * 34] : sh.vsum[nvec + j];
     if (work && lane < nvec) coef[lane] = (V)sh.hcol[lane];  // every warp the same values
     if (!work && owner && mode == ORTH_STEP) {
       if (!redo) {
@@ -649,7 +652,7 @@ __global__ void __launch_bounds__(kOneThreads, 1)
   }
   if (owner && tid == 0) ctl->bar_base = base + bars * gridDim.x;
   if (!redo) return;
-  reduce_sums(sh, part2, n2, gridDim.x);
+  reduce_sums(sh, part2, n2, gridDim.x, -1);
   if (warp == 0) second_column(sh, nvec, S.h2);
   __syncthreads();
   if (work && lane < nvec) coef[lane] = (V)sh.sum[lane];
@@ -1006,7 +1009,8 @@ __global__ void __launch_bounds__(kManyThreads, 1)
       if (givens && mode == ORTH_STEP) load_gram(sh.E, gram<V>(S), j);
       if (givens && mode != ORTH_STEP)
         for (int i = 0; i < 33; ++i) sh.E[i * 32 + lane] = V(0);
-      reduce_sums(sh, part1 + (int64_t)P.seg_slot[2 * s] * 64, n1, P.seg_slot[2 * s + 1]);
+      reduce_sums(sh, part1 + (int64_t)P.seg_slot[2 * s] * 64, n1, P.seg_slot[2 * s + 1],
+                  nvec + j);
       first_column(sh, j, mode, S, mode == ORTH_STEP);
       __syncthreads();
       if (warp == 0) {
@@ -1102,7 +1106,7 @@ __global__ void __launch_bounds__(kManyThreads, 1)
       SegState& S = st[s];
       if (mode != ORTH_FIN && S.act != 2) continue;
       __syncthreads();
-      reduce_sums(sh, part2 + (int64_t)P.seg_slot[2 * s] * 64, n2, P.seg_slot[2 * s + 1]);
+      reduce_sums(sh, part2 + (int64_t)P.seg_slot[2 * s] * 64, n2, P.seg_slot[2 * s + 1], -1);
       if (warp == 0) second_column(sh, nvec, S.h2);
       __syncthreads();
       if (warp == 0) {
