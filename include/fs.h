@@ -247,9 +247,9 @@ void fs_default_solve_opts(fs_solve_opts* opts);
  * NULL means the problem's state vector.  Synchronises.  stats may be NULL.
  * Returns FS_ERR_NOT_CONVERGED (with the best iterate kept) when max_iter or
  * max_refine is reached first, FS_ERR_NUMERIC on NaN/Inf, FS_ERR_TIMEOUT when
- * a wait inside a kernel has not ended after one second (the blocks of the
+ * a wait inside a kernel has not ended after its limit (the blocks of the
  * orthogonalisation kernel meet at barriers; the iterate is then undefined,
- * and the problem can be solved again).  fs_step, fs_step_picard,
+ * and the problem can be solved again from a new state; fs_set_wait_limit).  fs_step, fs_step_picard,
  * fs_solve_steady and the server report the status of their solves. */
 int fs_solve(fs_problem* prob, const fs_solve_opts* opts, double* x,
              fs_solve_stats* stats);
@@ -328,7 +328,7 @@ int fs_solve_steady(fs_problem* prob, const fs_solve_opts* opts, double nl_tol,
  * residual of rtol (checked every 8 iterations; FS_ERR_NOT_CONVERGED when
  * the true residual is above 100 rtol after max_iter iterations,
  * FS_ERR_TIMEOUT when a wait inside the solve's one kernel has not ended after
- * one second), whatever
+ * its limit), whatever
  * the problem's precision.  Needs a single problem with Dirichlet velocity on
  * the whole boundary and the pressure pin (FS_ERR_UNSUPPORTED otherwise).
  * per_step (host, nsteps entries, may be NULL).  Synchronises. */
@@ -339,6 +339,14 @@ typedef struct {
 } fs_ipcs_stats;
 int fs_step_ipcs(fs_problem* prob, int nsteps, double rtol, int max_iter,
                  fs_ipcs_stats* per_step);
+
+/* Limit, in nanoseconds, of every wait of a block for other blocks or for its
+ * copies inside the problem's orthogonalisation and CG kernels: 1e9 (one
+ * second) when the problem is created, 0 to 6e10; at 0 a wait ends at its first
+ * look.  A wait that runs out ends the call with FS_ERR_TIMEOUT; the time of a
+ * solve is not limited.  FS_ERR_BUSY while a step is in progress.
+ * Synchronises.  No counterpart in the paper. */
+int fs_set_wait_limit(fs_problem* prob, int64_t ns);
 
 /* Per-instance statistics of the last solve (host array, one entry per
  * instance). */

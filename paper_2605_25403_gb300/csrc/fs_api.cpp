@@ -198,6 +198,7 @@ struct fs_problem {
   double *ip_dA = nullptr, *ip_dM = nullptr, *ip_dK = nullptr, *ip_part = nullptr;
   double *ip_sc = nullptr, *ip_nrm = nullptr;
   CgCtl* ip_ctl = nullptr;
+  uint64_t wait_ns = kWaitNs;  // limit of the waits of its CG solves
   // SELL-32 values of the two velocity operators (P2/P1 problems)
   double *ip_sA = nullptr, *ip_sM = nullptr;
   uint8_t* ip_fixed = nullptr;
@@ -1325,7 +1326,7 @@ void finish_solve(fs_problem* P) {
   for (int s = 0; s < P->nseg; ++s)
     if (c.status[s] != FS_OK && c.rc == FS_OK) c.rc = c.status[s];
   if (c.rc == FS_ERR_TIMEOUT)
-    set_error("a wait inside a solver kernel did not end within a second");
+    set_error("a wait inside a solver kernel did not end within its limit");
   else if (c.rc != FS_OK)
     set_error("the solve did not reach rtol in every instance");
   c.phase = PH_DONE;
@@ -2577,7 +2578,7 @@ static int ipcs_cg(fs_problem* P, int which, const double* vals, const double* s
     op.ci = which == 1 ? m.ciK : m.ciA;
     op.v = vals;
     launch_cg_solve(m, which, op, rhs, x, dinv, P->ip_r, P->ip_z, P->ip_p, P->ip_p2, P->ip_q,
-                    P->ip_part, P->ip_ctl, rtol, max_iter, s);
+                    P->ip_part, P->ip_ctl, rtol, max_iter, P->wait_ns, s);
     FS_TRY(check_launch("ipcs cg"));
     CgCtl c;
     FS_CUDA(cudaMemcpyAsync(&c, P->ip_ctl, sizeof(c), cudaMemcpyDeviceToHost, s));
@@ -2585,7 +2586,7 @@ static int ipcs_cg(fs_problem* P, int which, const double* vals, const double* s
     *iters = c.iters;
     *relres = c.bb > 0 ? std::sqrt(c.rr / c.bb) : std::sqrt(c.rr);
     if (c.bad) {
-      set_error("a wait inside the CG kernel did not end within a second");
+      set_error("a wait inside the CG kernel did not end within its limit");
       return FS_ERR_TIMEOUT;
     }
     if (!std::isfinite(*relres)) return FS_ERR_NUMERIC;
@@ -2949,6 +2950,24 @@ int fs_profile_kernel(fs_problem* P, int kernel, int reps, double* avg_ms, doubl
   *avg_ms = ms / reps;
   *alg_bytes = bytes;
   if (kernel == FS_KERNEL_ASSEMBLE_CONV) FS_TRY(assemble_impl(P, P->t + P->desc.dt));
+  return FS_OK;
+}
+
+int fs_set_wait_limit(fs_problem* P, int64_t ns) {
+  if (!P || ns < 0 || ns > (int64_t)60000000000) {
+    set_error("fs_set_wait_limit: null problem, or a limit outside 0 to 60 s");
+    return FS_ERR_INVALID_ARG;
+  }
+  if (P->ctx.phase != PH_IDLE && P->ctx.phase != PH_DONE) {
+    set_error("fs_set_wait_limit: a step is in progress");
+    return FS_ERR_BUSY;
+  }
+  const uint64_t v = (uint64_t)ns;
+  for (KCtl* c : {P->p64.kr.ctl, P->p32.kr.ctl})
+    if (c)
+      FS_CUDA(cudaMemcpyAsync(&c->wait_ns, &v, sizeof(v), cudaMemcpyHostToDevice, P->stream));
+  FS_CUDA(cudaStreamSynchronize(P->stream));
+  P->wait_ns = v;
   return FS_OK;
 }
 

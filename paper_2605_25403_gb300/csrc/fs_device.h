@@ -29,8 +29,9 @@ void count_launches(int64_t n);
 // problem's schedule by the API entry points.
 bool launch_overlap();
 
-// Limit of a wait inside a kernel: one second.  A kernel whose wait runs out
-// marks its result and returns, and the call reports FS_ERR_TIMEOUT.
+// Limit of a wait inside a kernel: one second (fs_set_wait_limit changes a
+// problem's).  A kernel whose wait runs out marks its result and returns, and
+// the call reports FS_ERR_TIMEOUT.
 constexpr uint64_t kWaitNs = 1000000000ull;
 
 #ifdef __CUDACC__
@@ -556,7 +557,7 @@ struct CgOp {
 void launch_cg_solve(const DMesh& m, int which, const CgOp& op, const double* rhs, double* x,
                      const double* dinv, double* r, double* z, double* p, double* p2,
                      double* q, double* part, CgCtl* ctl, double rtol, int max_iter,
-                     cudaStream_t s);
+                     uint64_t wait_ns, cudaStream_t s);
 // The V-cycle-preconditioned pressure stage, a kernel per step; sc (4 doubles
 // on the device): rz, alpha, beta, rr.
 void launch_cg_init(int64_t n, const double* rhs, const double* y, const double* dinv, double* r,

@@ -813,7 +813,7 @@ void launch_cg_dots_flex(int64_t n, const uint8_t* fixed, const double* r, const
 void launch_cg_solve(const DMesh& m, int which, const CgOp& op, const double* rhs, double* x,
                      const double* dinv, double* r, double* z, double* p, double* p2,
                      double* q, double* part, CgCtl* ctl, double rtol, int max_iter,
-                     cudaStream_t s) {
+                     uint64_t wait_ns, cudaStream_t s) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -837,7 +837,7 @@ void launch_cg_solve(const DMesh& m, int which, const CgOp& op, const double* rh
   cfg.numAttrs = 1;
   auto go = [&](auto k) {
     cudaLaunchKernelEx(&cfg, k, op, rhs, x, dinv, r, z, p, p2, q, part, ctl, rtol, max_iter,
-                       kWaitNs);
+                       wait_ns);
   };
   if (which == 1) go(wide ? k_cg_solve<1, 8> : k_cg_solve<1, 1>);
   else if (m.dim == 2) go(wide ? k_cg_solve<2, 8> : k_cg_solve<2, 1>);

@@ -183,6 +183,8 @@ _lib.fs_launch_count.restype = _i64
 _lib.fs_launch_count.argtypes = []
 _lib.fs_profile_kernel.restype = _int
 _lib.fs_profile_kernel.argtypes = [_vp, _int, _int, _P(_d), _P(_d)]
+_lib.fs_set_wait_limit.restype = _int
+_lib.fs_set_wait_limit.argtypes = [_vp, _i64]
 _lib.fs_get_schedule.restype = _int
 _lib.fs_get_schedule.argtypes = [_vp, _P(fs_schedule)]
 _lib.fs_autotune_smoother.restype = _int
@@ -206,7 +208,7 @@ EXPORTED = ["fs_mesh_create", "fs_mesh_destroy", "fs_dof_map", "fs_problem_creat
             "fs_step_begin", "fs_step_poll", "fs_instance_stats", "fs_server_create",
             "fs_server_destroy", "fs_server_submit", "fs_server_progress",
             "fs_server_pop_completed", "fs_server_take_state", "fs_server_status",
-            "fs_server_estimate_bytes", "fs_get_schedule", "fs_set_schedule", "fs_autotune",
+            "fs_server_estimate_bytes", "fs_set_wait_limit", "fs_get_schedule", "fs_set_schedule", "fs_autotune",
             "fs_autotune_smoother",
             "fs_step_picard", "fs_solve_steady", "fs_step_ipcs", "fs_problem_create_p3",
             "fs_problem_sizes"]
@@ -502,6 +504,11 @@ def fs_csr_residual_norm_noalloc(rowptr, col, val, x, b, stream=None, n=None):
 
 def fs_launch_count():
     return int(_lib.fs_launch_count())
+
+
+def fs_set_wait_limit(prob, seconds):
+    """Limit of the waits inside the problem's kernels (1 s by default)."""
+    _check(_lib.fs_set_wait_limit(prob, int(round(1e9 * seconds))), "fs_set_wait_limit")
 
 
 def fs_get_schedule(prob):
